@@ -172,6 +172,8 @@ struct tc_graph {
     uint64_t* tnew = nullptr;   // per-vertex accumulator in new labels, n
     unsigned* tlow = nullptr;   // 32-bit per-task shares (per-vertex counts), n, on demand
     size_t tlow_bytes = 0;
+    size_t zero_bytes = 0;      // [counters | comp_totals | tnew | tlow (small graphs)] are one range
+    bool tlow_in_arena = false;
 
     // instrumentation of a host-input preprocessing (set by tc_triangles):
     // an event recorded on the stream once the pairs are uploaded, and the

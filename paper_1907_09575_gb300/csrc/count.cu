@@ -41,7 +41,8 @@ namespace {
 #define TC_LARGE_MINB 4        // CTAs per SM the CTA kernel's registers must allow
 #endif
 
-constexpr int kGrab = 4;          // warp units popped per queue access
+constexpr int kGrab = 4;          // warp units popped per queue access ...
+constexpr int kGrabMin = 8;       // ... when every warp gets this many or more, else one
 constexpr int kEmpty = -1;
 #ifndef TC_UNROLL
 #define TC_UNROLL 4
@@ -902,7 +903,8 @@ template <bool PV, bool MERGE, bool WIN, bool BUCKETS>
 __global__ void __launch_bounds__(256, TC_LARGE_MINB)
     k_count(const GraphView* __restrict__ views, const Unit* __restrict__ large, int64_t nlarge,
             const Unit* __restrict__ small, int64_t nsmall, int slice_max, int table_mode,
-            int merge_max, unsigned* tlow, unsigned long long* __restrict__ ctr) {
+            int merge_max, int grab, unsigned* tlow,
+            unsigned long long* __restrict__ ctr) {
     extern __shared__ __align__(16) unsigned smem[];
     __shared__ long long s_unit;
     __shared__ int s_ctl[4];
@@ -951,10 +953,10 @@ __global__ void __launch_bounds__(256, TC_LARGE_MINB)
     uint64_t staged = 0;
     while (true) {
         long long u0 = 0;
-        if (lane == 0) u0 = (long long)atomicAdd(&ctr[CTR_SMALL_HEAD], (unsigned long long)kGrab);
+        if (lane == 0) u0 = (long long)atomicAdd(&ctr[CTR_SMALL_HEAD], (unsigned long long)grab);
         u0 = __shfl_sync(0xffffffffu, u0, 0);
         if (u0 >= nsmall) break;
-        const int64_t u1 = min64(u0 + kGrab, nsmall);
+        const int64_t u1 = min64(u0 + grab, nsmall);
         for (int64_t u = u0; u < u1; ++u) {
             const Unit U = small[u];
             const GraphView G = views[U.g];
@@ -1151,7 +1153,7 @@ size_t count_smem_bytes(bool pv, int threads, int unit_tasks) {
            sizeof(unsigned short) * (size_t)unit_tasks;
 }
 
-using CountKernel = void (*)(const GraphView*, const Unit*, int64_t, const Unit*, int64_t, int, int, int,
+using CountKernel = void (*)(const GraphView*, const Unit*, int64_t, const Unit*, int64_t, int, int, int, int,
                             unsigned*, unsigned long long*);
 
 // the count kernel instance for a launch: per-vertex or totals, with or
@@ -1180,8 +1182,10 @@ CountLaunch prepare_count(const UnitLists& L, const tc_tuning& t, bool pv, bool 
     int per_sm = 0;
     TC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, c.threads, c.smem));
     per_sm = std::max(per_sm, 1);
+    const int64_t warps = (int64_t)num_sms() * per_sm * (c.threads / 32);
+    c.grab = L.nsmall < kGrabMin * warps ? 1 : kGrab;
     const int64_t want =
-        L.nlarge + (L.nsmall + kGrab * (c.threads / 32) - 1) / (kGrab * (c.threads / 32));
+        L.nlarge + (L.nsmall + c.grab * (c.threads / 32) - 1) / (c.grab * (c.threads / 32));
     c.grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)num_sms() * per_sm, want));
     return c;
 }
@@ -1191,7 +1195,7 @@ void launch_count_raw(const CountLaunch& c, const GraphView* views_dev, const Un
     if (L.nlarge + L.nsmall == 0) return;
     auto kern = count_kernel(c.pv, c.merge, c.win, c.buckets);
     kern<<<c.grid, c.threads, c.smem, st>>>(views_dev, L.large, L.nlarge, L.small, L.nsmall,
-                                            t.slice_max, t.table_mode, t.merge_max_outdeg, tlow, ctr);
+                                            t.slice_max, t.table_mode, t.merge_max_outdeg, c.grab, tlow, ctr);
     TC_LAUNCH_CHECK();
 }
 
@@ -1221,8 +1225,10 @@ void count_components(tc_graph* g, const tc_tuning& t, uint64_t* comp_totals_dev
                       cudaStream_t st) {
     const tc_tuning tt = clamp_tuning(size_tuning(t, g->m));
     if (!tuning_equal(tt, g->units_tuning)) build_units(g, tt, st);
-    TC_CUDA(cudaMemsetAsync(g->counters, 0, sizeof(unsigned long long) * CTR_COUNT, st));
-    TC_CUDA(cudaMemsetAsync(g->comp_totals, 0, sizeof(unsigned long long) * (size_t)g->num_comps, st));
+    // counters and component totals lie next to each other
+    TC_CUDA(cudaMemsetAsync(g->counters, 0,
+                            (size_t)(reinterpret_cast<char*>(g->comp_totals + g->num_comps) -
+                                     reinterpret_cast<char*>(g->counters)), st));
     UnitLists L;
     L.large = g->large_units;
     L.small = g->small_units;
@@ -1239,12 +1245,12 @@ void count(tc_graph* g, const tc_tuning& t, uint64_t* total_dev, uint64_t* per_v
     const tc_tuning tt = clamp_tuning(size_tuning(t, g->m));
     if (!tuning_equal(tt, g->units_tuning)) build_units(g, tt, st);
     const bool pv = per_vertex_dev != nullptr;
-    TC_CUDA(cudaMemsetAsync(g->counters, 0, sizeof(unsigned long long) * CTR_COUNT, st));
-    if (pv && g->n > 0) TC_CUDA(cudaMemsetAsync(g->tnew, 0, sizeof(uint64_t) * (size_t)g->n, st));
+    // the counters, and with per-vertex counts the accumulators behind them
+    TC_CUDA(cudaMemsetAsync(g->counters, 0, pv ? g->zero_bytes : sizeof(unsigned long long) * CTR_COUNT, st));
     // a task's share is at most C(max |U_i|, 2): 32-bit counters when that fits
     const uint64_t dmax = (uint64_t)g->stats.max_outdeg;
     const bool tlow32 = TC_TLOW32 && pv && g->n > 0 && dmax * (dmax - (dmax > 0)) / 2 < (1ull << 32);
-    if (tlow32) {
+    if (tlow32 && !g->tlow_in_arena) {
         if (!g->tlow) {
             g->tlow_bytes = sizeof(unsigned) * (size_t)g->n;
             g->tlow = static_cast<unsigned*>(g->alloc.get(g->tlow_bytes));

@@ -624,6 +624,63 @@ __global__ void k_comp_new(const int32_t* __restrict__ perm, int64_t n, const in
 
 }  // namespace
 
+void graph_arena(tc_graph* g, int64_t cap_m, bool off64, int32_t num_comps) {
+    const size_t n = (size_t)g->n, nv = std::max<size_t>(n, 1), m = (size_t)std::max<int64_t>(cap_m, 1);
+    const bool low = g->n <= kBuildMaxPairs;   // larger graphs take tlow when they need it
+    size_t need = 0;
+    auto take = [&](size_t bytes) {
+        const size_t at = need;
+        need += align_up(bytes);
+        return at;
+    };
+    const size_t o_off = take((off64 ? 8 : 4) * (n + 1)), o_adj = take(4 * m), o_perm = take(4 * nv);
+    const size_t o_loff = take(8 * (n + 1)), o_tasks = take(sizeof(Task) * m);
+    const size_t o_view = take(sizeof(GraphView)), o_vc = take(sizeof(GraphView));
+    const size_t o_comp = take(num_comps > 0 ? 4 * nv : 0);
+    const size_t o_ctr = take(sizeof(unsigned long long) * CTR_COUNT);
+    const size_t o_ctot = take(8 * (size_t)std::max(num_comps, 0));
+    const size_t o_tnew = take(8 * nv), o_tlow = take(low ? 4 * nv : 0);
+    g->off64 = off64;
+    g->arena_bytes = need;
+    g->arena = g->alloc.get(need);
+    char* a = static_cast<char*>(g->arena);
+    g->off = a + o_off;
+    g->adj = reinterpret_cast<int32_t*>(a + o_adj);
+    g->perm = reinterpret_cast<int32_t*>(a + o_perm);
+    g->loff = reinterpret_cast<int64_t*>(a + o_loff);
+    g->tasks = reinterpret_cast<Task*>(a + o_tasks);
+    g->view = reinterpret_cast<GraphView*>(a + o_view);
+    g->view_comp = reinterpret_cast<GraphView*>(a + o_vc);
+    g->counters = reinterpret_cast<unsigned long long*>(a + o_ctr);
+    g->tnew = reinterpret_cast<uint64_t*>(a + o_tnew);
+    g->zero_bytes = need - o_ctr;
+    if (low) {
+        g->tlow = reinterpret_cast<unsigned*>(a + o_tlow);
+        g->tlow_in_arena = true;
+    }
+    if (num_comps > 0) {
+        g->comp = reinterpret_cast<int32_t*>(a + o_comp);
+        g->comp_totals = reinterpret_cast<unsigned long long*>(a + o_ctot);
+        g->num_comps = num_comps;
+    }
+}
+
+void graph_views(const tc_graph* g, GraphView* v, GraphView* vc) {
+    *v = GraphView{};
+    v->off = g->off;
+    v->adj = g->adj;
+    v->loff = g->loff;
+    v->tasks = g->tasks;
+    v->tnew = reinterpret_cast<unsigned long long*>(g->tnew);
+    v->total = g->counters + CTR_TOTAL;
+    v->n = g->n;
+    v->off64 = g->off64 ? 1 : 0;
+    *vc = *v;
+    vc->tnew = nullptr;
+    vc->comp = g->comp;
+    vc->comp_totals = g->comp_totals;
+}
+
 void preprocess(tc_graph* g, const int32_t* src_in, const int32_t* dst_in, int64_t P,
                 uint32_t flags, cudaStream_t st) {
     preprocess_with_components(g, src_in, dst_in, P, flags, nullptr, 0, st);
@@ -701,6 +758,11 @@ void preprocess_with_components(tc_graph* g, const int32_t* src_in, const int32_
         dst = hdst.get();
     }
     if (g->ev_uploaded) TC_CUDA(cudaEventRecord(g->ev_uploaded, st));
+
+    if (build_takes(P, n)) {
+        build_graph(g, src, dst, P, flags, vpre_host, num_comps, st);
+        return;
+    }
 
     Buf<int> scal(al, 8);   // [0] err, [1] max degree, [2] max out-degree, [3] heavy vertices
     TC_CUDA(cudaMemsetAsync(scal.get(), 0, 8 * sizeof(int), st));
@@ -814,37 +876,7 @@ void preprocess_with_components(tc_graph* g, const int32_t* src_in, const int32_
                                                                          : (m >= (int64_t)0x7fffffff);
     const size_t ob = g->off64 ? 8 : 4;
 
-    // arena: off, adj, perm, loff, tasks (capacity m), counters, tnew
-    size_t sz_off = align_up(ob * (size_t)(n + 1)), sz_adj = align_up(4 * (size_t)std::max<int64_t>(m, 1));
-    size_t sz_perm = align_up(4 * (size_t)std::max<int64_t>(n, 1));
-    size_t sz_loff = align_up(8 * (size_t)(n + 1));
-    size_t sz_tasks = align_up(sizeof(Task) * (size_t)std::max<int64_t>(m, 1));
-    size_t sz_ctr = align_up(sizeof(unsigned long long) * CTR_COUNT) + align_up(sizeof(GraphView));
-    size_t sz_tnew = align_up(8 * (size_t)std::max<int64_t>(n, 1));
-    size_t sz_comp = num_comps > 0 ? align_up(4 * (size_t)std::max<int64_t>(n, 1)) : 0;
-    size_t sz_ctot = num_comps > 0 ? align_up(8 * (size_t)num_comps) : 0;
-    sz_ctr += align_up(sizeof(GraphView));
-    g->arena_bytes = sz_off + sz_adj + sz_perm + sz_loff + sz_tasks + sz_ctr + sz_tnew + sz_comp + sz_ctot;
-    g->arena = al.get(g->arena_bytes);
-    char* a = static_cast<char*>(g->arena);
-    g->off = a; a += sz_off;
-    g->adj = reinterpret_cast<int32_t*>(a); a += sz_adj;
-    g->perm = reinterpret_cast<int32_t*>(a); a += sz_perm;
-    g->loff = reinterpret_cast<int64_t*>(a); a += sz_loff;
-    g->tasks = reinterpret_cast<Task*>(a); a += sz_tasks;
-    g->counters = reinterpret_cast<unsigned long long*>(a);
-    g->view = reinterpret_cast<GraphView*>(a + align_up(sizeof(unsigned long long) * CTR_COUNT));
-    g->view_comp = reinterpret_cast<GraphView*>(a + align_up(sizeof(unsigned long long) * CTR_COUNT) +
-                                                align_up(sizeof(GraphView)));
-    a += sz_ctr;
-    g->tnew = reinterpret_cast<uint64_t*>(a);
-    a += sz_tnew;
-    if (num_comps > 0) {
-        g->comp = reinterpret_cast<int32_t*>(a);
-        a += sz_comp;
-        g->comp_totals = reinterpret_cast<unsigned long long*>(a);
-        g->num_comps = num_comps;
-    }
+    graph_arena(g, m, g->off64, num_comps);
 
     // a4 relabel
     if (n > 0) {
@@ -1037,22 +1069,11 @@ void preprocess_with_components(tc_graph* g, const int32_t* src_in, const int32_
             }
         TC_LAUNCH_CHECK();
     }
-    // the device view the count kernel reads (pageable sources: staged on return)
+    // the device views the count kernel reads (pageable sources: staged on return)
     {
-        GraphView v{};
-        v.off = g->off;
-        v.adj = g->adj;
-        v.loff = g->loff;
-        v.tasks = g->tasks;
-        v.tnew = reinterpret_cast<unsigned long long*>(g->tnew);
-        v.total = g->counters + CTR_TOTAL;
-        v.n = n;
-        v.off64 = g->off64 ? 1 : 0;
+        GraphView v, vc;
+        graph_views(g, &v, &vc);
         TC_CUDA(cudaMemcpyAsync(g->view, &v, sizeof(v), cudaMemcpyHostToDevice, st));
-        GraphView vc = v;
-        vc.tnew = nullptr;
-        vc.comp = g->comp;
-        vc.comp_totals = g->comp_totals;
         TC_CUDA(cudaMemcpyAsync(g->view_comp, &vc, sizeof(vc), cudaMemcpyHostToDevice, st));
     }
 

@@ -35,6 +35,22 @@ void preprocess(tc_graph* g, const int32_t* src, const int32_t* dst, int64_t P, 
 void preprocess_with_components(tc_graph* g, const int32_t* src, const int32_t* dst, int64_t P,
                                 uint32_t flags, const int64_t* vpre_host, int32_t num_comps,
                                 cudaStream_t st);
+// The graph's device arena for up to cap_m edges (offsets, columns, labels,
+// tasks, counters, accumulators, components), and its views into it.
+void graph_arena(tc_graph* g, int64_t cap_m, bool off64, int32_t num_comps);
+void graph_views(const tc_graph* g, GraphView* v, GraphView* vc);
+
+// Preprocessing of graphs of up to kBuildMaxPairs pairs in one persistent
+// kernel (build.cu).
+constexpr int64_t kBuildMaxPairs = 1ll << 24;
+// up to here the arena is sized by the pairs and the host waits once (a round
+// trip with its allocations and launch costs ~25 us, a tenth of a call of 2^20
+// pairs); beyond, by the edges
+constexpr int64_t kBuildOnePairs = 1ll << 22;
+bool build_takes(int64_t P, int64_t n);
+void build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64_t P, uint32_t flags,
+                 const int64_t* vpre_host, int32_t num_comps, cudaStream_t st);
+
 // Unit lists over the graphs of a view table (one graph, or a batch).
 struct UnitLists {
     void* mem = nullptr;
@@ -69,6 +85,7 @@ struct CountLaunch {
     unsigned grid = 1;
     int threads = 256;
     size_t smem = 0;
+    int grab = 1;         // warp units popped per queue access
     bool pv = false;
     bool merge = false;   // the instance with the search path for short pivot rows
     bool win = false;     // the instance that counts one tile (a window of rows)

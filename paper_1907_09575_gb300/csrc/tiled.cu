@@ -103,10 +103,12 @@ void graph_offload(tc_graph* g, cudaStream_t st) {
     }
     g->alloc.stream = st;
     if (g->units_mem) g->alloc.put(g->units_mem, g->units_bytes);
-    if (g->tlow) g->alloc.put(g->tlow, g->tlow_bytes);
+    if (g->tlow && !g->tlow_in_arena) g->alloc.put(g->tlow, g->tlow_bytes);
     if (g->arena) g->alloc.put(g->arena, g->arena_bytes);
     g->units_mem = nullptr;
     g->tlow = nullptr;
+    g->tlow_in_arena = false;
+    g->zero_bytes = 0;
     g->arena = nullptr;
     g->off = nullptr;
     g->adj = nullptr;
