@@ -64,12 +64,15 @@ void set_tuning(tc_batch* b, const tc_tuning& t) {
     TC_CUDA(cudaStreamSynchronize(b->cap));
     b->tuning = tt;
     const CountLaunch c = prepare_count(b->units, tt, false);
+    prepare_mid();
     TC_CUDA(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
     cudaError_t e1 = cudaMemsetAsync(b->ctr, 0, sizeof(unsigned long long) * CTR_COUNT, b->cap);
     cudaError_t e2 = cudaMemsetAsync(b->totals, 0, sizeof(uint64_t) * (size_t)b->num, b->cap);
     bool launched = true;
     try {
         launch_count_raw(c, b->views, b->units, tt, b->ctr, b->cap);
+        launch_mid(b->views, b->units, tt, false, b->ctr, b->cap, nullptr, false);
+        launch_zone(b->views, b->units, false, b->ctr, b->cap, nullptr, false);
     } catch (const Error&) {
         launched = false;
     }
@@ -197,15 +200,10 @@ tc_status tc_batch_create(const tc_graph* const* graphs, int32_t num, const tc_t
         std::vector<int64_t> hp(num + 1, 0);
         for (int32_t k = 0; k < num; ++k) {
             const tc_graph* g = b->graphs[k];
-            GraphView v{};
-            v.off = g->off;
-            v.adj = g->adj;
-            v.loff = g->loff;
-            v.tasks = g->tasks;
+            GraphView v, vc;
+            graph_views(g, &v, &vc);
             v.tnew = nullptr;
             v.total = reinterpret_cast<unsigned long long*>(b->totals + b->slot[k]);
-            v.n = g->n;
-            v.off64 = g->off64 ? 1 : 0;
             hv[k] = v;
             hp[k + 1] = hp[k] + g->n;
         }
@@ -300,12 +298,15 @@ tc_status tc_batch_get_count_stats(const tc_batch* b, tc_count_stats* out, void*
     TC_CUDA(cudaMemcpyAsync(tot.data(), b->totals, sizeof(uint64_t) * b->num, cudaMemcpyDeviceToHost, st));
     TC_CUDA(cudaStreamSynchronize(st));
     out->triangles = std::accumulate(tot.begin(), tot.end(), (uint64_t)0);
+    uint64_t covered = 0;   // entries counted as zone bits
+    for (const tc_graph* g : b->graphs) covered += g->covered;
     for (int k = 0; k < 2; ++k) {
         out->units[k] = c[CTR_UNITS + k];
         out->tasks[k] = c[CTR_TASKS + k];
         out->probes[k] = c[CTR_PROBES + k];
         out->staged[k] = c[CTR_STAGED + k];
     }
+    out->probes[1] += covered;
     TC_API_END
 }
 

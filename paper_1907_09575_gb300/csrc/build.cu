@@ -33,6 +33,7 @@
 
 #include "common.cuh"
 #include "tc_internal.cuh"
+#include "zone.cuh"
 
 namespace tc {
 namespace {
@@ -59,7 +60,9 @@ struct Tally {
     int nmed, nlong;         // listed rows
     int med_head;
     unsigned long long m, tasks, probes, probes_ijk;
-    long long nsmall, nlarge;
+    long long nsmall, nlarge, nzone;
+    unsigned long long covered;
+    unsigned nblocks, pad;
 };
 
 struct BuildArgs {
@@ -82,7 +85,7 @@ struct BuildArgs {
     int tcopies;             // then the first slot of each copy's tasks
     uint32_t *ord0, *ord1;   // vertices between the relabel's passes; later the listed rows
     unsigned* hist;          // nchunks x 256
-    long long* sums;         // 4 x nchunks
+    long long* sums;         // 5 x nchunks
     uint2* pairs;            // oriented pairs (in the table's memory)
     uint32_t* place;         // place of a pair in its row; later of an edge among its pivot's tasks
     uint32_t* row;           // row of each edge
@@ -92,9 +95,12 @@ struct BuildArgs {
     int64_t* loff;
     Task* tasks;
     int32_t* comp;
+    uint2* zrow;             // dense zones (zcap > 0)
+    uint32_t *zbits, *zowner;
+    int64_t zcap;
     GraphView view, view_comp;
     GraphView *view_at, *view_comp_at;
-    Unit *small, *large;
+    Unit *small, *large, *zone;
     int small_max, warp_tasks, cta_tasks, slice_max;
 };
 
@@ -438,6 +444,7 @@ __device__ void offsets_sum(const BuildArgs& a) {
     unsigned long long probes = 0, ijk = 0;
     int mx = 0;
     for (int64_t r = c0 + threadIdx.x; r < c1; r += kBT) {
+        if (a.zcap > 0) a.zrow[r] = make_uint2(0, 0);
         const long long d = a.dplus[r], din = a.degn[r] - d;
         s += d;
         mx = max(mx, (int)d);
@@ -688,25 +695,27 @@ __device__ void phase_sort(const BuildArgs& a, uint32_t* smem) {
 
 // --- tasks and units ----------------------------------------------------------
 __device__ __forceinline__ void unit_counts(const BuildArgs& a, long long dp, long long nt, long long& small,
-                                            long long& large) {
+                                            long long& large, long long& zone) {
     small = large = 0;
+    zone = a.zcap > 0 && dp > kZoneMinPivot ? (nt + kZoneTasks - 1) / kZoneTasks : 0;
     if (dp > 0 && nt > 0) {
         if (dp <= a.small_max) small = (nt + a.warp_tasks - 1) / a.warp_tasks;
-        else large = ((dp + a.slice_max - 1) / a.slice_max) * ((nt + a.cta_tasks - 1) / a.cta_tasks);
+        else if (zone == 0 || dp > kMidMaxOutdeg) large = ((dp + a.slice_max - 1) / a.slice_max) * ((nt + a.cta_tasks - 1) / a.cta_tasks);
     }
 }
 
 __device__ void tasks_sum(const BuildArgs& a) {
     if ((int)blockIdx.x >= a.nchunks) return;
     const int64_t c0 = (int64_t)blockIdx.x * a.chunk, c1 = min64(c0 + a.chunk, a.n);
-    long long t = 0, us = 0, ul = 0, total;
+    long long t = 0, us = 0, ul = 0, uz = 0, total;
     for (int64_t r = c0 + threadIdx.x; r < c1; r += kBT) {
-        long long x, y, nt = 0;
+        long long x, y, z, nt = 0;
         for (int c = 0; c < a.tcopies; ++c) nt += a.tcur[c * a.n + r];
-        unit_counts(a, a.dplus[r], nt, x, y);
+        unit_counts(a, a.dplus[r], nt, x, y, z);
         t += nt;
         us += x;
         ul += y;
+        uz += z;
     }
     long long* s = a.sums + a.nchunks;   // the row sums may still be read by slower blocks
     block_scan(t, &total);
@@ -720,6 +729,25 @@ __device__ void tasks_sum(const BuildArgs& a) {
     if (threadIdx.x == 0) {
         s[2 * a.nchunks + blockIdx.x] = total;
         if (total) atomicAdd(reinterpret_cast<unsigned long long*>(&a.tally->nlarge), (unsigned long long)total);
+    }
+    block_scan(uz, &total);
+    if (threadIdx.x == 0) {
+        s[3 * a.nchunks + blockIdx.x] = total;
+        if (total) atomicAdd(reinterpret_cast<unsigned long long*>(&a.tally->nzone), (unsigned long long)total);
+    }
+}
+
+// --- zones: the bit blocks of the listed rows, a warp each --------------------
+__device__ void phase_zones(const BuildArgs& a, uint32_t* smem) {
+    if (a.zcap == 0) return;
+    const int w = threadIdx.x >> 5;
+    uint32_t* buf = smem + w * kZoneWords;
+    const int nmed = a.tally->nmed, all = nmed + a.tally->nlong;
+    for (int x = blockIdx.x * kBW + w; x < all; x += gridDim.x * kBW) {
+        const uint32_t r = x < nmed ? a.ord0[x] : a.ord1[x - nmed];
+        const int64_t rb = row_begin(a, r);
+        zone_row(a.adj, rb, (int)(row_begin(a, (int64_t)r + 1) - rb), r, a.n, a.zrow, a.zbits, a.zowner, a.zcap,
+                 &a.tally->nblocks, buf);
     }
 }
 
@@ -739,11 +767,13 @@ __device__ void tasks_offsets(const BuildArgs& a) {
         long long run = carry + block_scan(s, &total);
         carry += total;
         if (r < c1) {
+            // the first slots, with the pivot's part in the zones in the top bit
+            const int32_t big = a.zcap > 0 && a.dplus[r] > kZoneMinPivot ? (int32_t)0x80000000 : 0;
             a.loff[r] = run;
 #pragma unroll
             for (int c = 0; c < kTaskCopies; ++c)
                 if (c < a.tcopies) {
-                    a.tcur[c * a.n + r] = (int32_t)run;
+                    a.tcur[c * a.n + r] = (int32_t)run | big;
                     run += d[c];
                 }
         }
@@ -757,10 +787,12 @@ __device__ void tasks_offsets(const BuildArgs& a) {
 __device__ void tasks_write(const BuildArgs& a) {
     const int64_t T = (int64_t)gridDim.x * kBT, t = (int64_t)blockIdx.x * kBT + threadIdx.x;
     const int64_t m = row_begin(a, a.n);
+    unsigned long long cut = 0;
     for (int64_t base = t; base < m; base += kBItems * T) {
         uint32_t i[kBItems], j[kBItems], at[kBItems];
         int len[kBItems];
         int32_t slot[kBItems];
+        uint2 zr[kBItems];
 #pragma unroll
         for (int u = 0; u < kBItems; ++u) {
             const int64_t e = base + u * T;
@@ -777,18 +809,22 @@ __device__ void tasks_write(const BuildArgs& a) {
             if (e < m) {
                 len[u] = (int)(row_begin(a, (int64_t)i[u] + 1) - e - 1);
                 slot[u] = a.tcur[task_counter(a, i[u], j[u])];
+                zr[u] = a.zcap > 0 ? a.zrow[i[u]] : make_uint2(0, 0);
             }
         }
 #pragma unroll
         for (int u = 0; u < kBItems; ++u)
             if (len[u] > 0) {
                 Task x;
-                x.start = base + u * T + 1;
-                x.len = len[u];
+                x.start = (uint32_t)(base + u * T + 1);
+                x.len = zone_cut(zr[u], slot[u] < 0, base + u * T, len[u], &x.zone);
                 x.i = (int32_t)i[u];
-                a.tasks[(int64_t)slot[u] + at[u]] = x;
+                cut += (unsigned)(len[u] - x.len);
+                a.tasks[(int64_t)(slot[u] & 0x7fffffff) + at[u]] = x;
             }
     }
+    cut = warp_sum(cut);
+    if ((threadIdx.x & 31) == 0 && cut) atomicAdd(&a.tally->covered, cut);
 }
 
 __device__ __forceinline__ void put_unit(const BuildArgs& a, int64_t j, bool small, long long at, int64_t q,
@@ -823,21 +859,24 @@ __device__ void phase_units(const BuildArgs& a) {
     const int64_t c0 = (int64_t)blockIdx.x * a.chunk, c1 = min64(c0 + a.chunk, a.n);
     long long cs = block_sum(a.sums + 2 * a.nchunks, blockIdx.x);
     long long cl = block_sum(a.sums + 3 * a.nchunks, blockIdx.x);
-    const long long ns = a.tally->nsmall, nl = a.tally->nlarge;
+    long long cz = block_sum(a.sums + 4 * a.nchunks, blockIdx.x);
+    const long long ns = a.tally->nsmall, nl = a.tally->nlarge, nz = a.tally->nzone;
     for (int64_t t0 = c0; t0 < c1; t0 += kBT) {
         const int64_t j = t0 + threadIdx.x;
-        long long us = 0, ul = 0, ts, tl;
+        long long us = 0, ul = 0, uz = 0, ts, tl, tz;
         int64_t b0 = 0, b1 = 0, slices = 1;
         if (j < c1) {
             const int64_t dp = row_begin(a, j + 1) - row_begin(a, j);
             b0 = a.loff[j];
             b1 = a.loff[j + 1];
-            unit_counts(a, dp, b1 - b0, us, ul);
+            unit_counts(a, dp, b1 - b0, us, ul, uz);
             slices = (dp + a.slice_max - 1) / a.slice_max;
         }
         const long long xs = cs + block_scan(us, &ts), xl = cl + block_scan(ul, &tl);
+        const long long az = nz - uz - (cz + block_scan(uz, &tz));
         cs += ts;
         cl += tl;
+        cz += tz;
         const bool small = us > 0;
         const long long count = us + ul;
         const long long at = small ? ns - xs - us : nl - xl - ul;
@@ -852,6 +891,16 @@ __device__ void phase_units(const BuildArgs& a) {
             const int64_t s = __shfl_sync(0xffffffffu, slices, o), jj = __shfl_sync(0xffffffffu, j, o);
             const bool sm = __shfl_sync(0xffffffffu, (int)small, o);
             for (int64_t q = lane; q < c; q += 32) put_unit(a, jj, sm, p, q, s, x0, x1);
+        }
+        unsigned zoned = __ballot_sync(0xffffffffu, uz > 0);
+        while (zoned) {
+            const int o = __ffs(zoned) - 1;
+            zoned &= zoned - 1;
+            const long long c = __shfl_sync(0xffffffffu, uz, o), p = __shfl_sync(0xffffffffu, az, o);
+            const int64_t x0 = __shfl_sync(0xffffffffu, b0, o), x1 = __shfl_sync(0xffffffffu, b1, o);
+            const int64_t jj = __shfl_sync(0xffffffffu, j, o);
+            for (int64_t q = lane; q < c; q += 32)
+                a.zone[p + q] = Unit{(int32_t)jj, 0, 0, 0, x0 + q * kZoneTasks, min64(x0 + (q + 1) * kZoneTasks, x1)};
         }
     }
 }
@@ -891,6 +940,7 @@ __global__ void __launch_bounds__(kBT, kBlocksPerSm) k_build(const __grid_consta
         phase_sort(a, smem);
         if (!grid.sync()) return;
         tasks_sum(a);
+        phase_zones(a, smem);
         if (!grid.sync()) return;
         tasks_offsets(a);
         if (!grid.sync()) return;
@@ -933,7 +983,7 @@ void build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64_t P,
         return at;
     };
     const size_t o_tally = take(sizeof(Tally)), o_vpre = take(8 * (size_t)(num_comps + 1));
-    const size_t o_hist = take(4 * 256 * (size_t)a.nchunks), o_sums = take(8 * 4 * (size_t)a.nchunks);
+    const size_t o_hist = take(4 * 256 * (size_t)a.nchunks), o_sums = take(8 * 5 * (size_t)a.nchunks);
     const size_t o_deg = take(4 * nv), o_degn = take(4 * nv), o_dplus = take(4 * nv), o_tcur = take(4 * nv * (size_t)a.tcopies);
     const size_t o_ord0 = take(4 * nv), o_ord1 = take(4 * nv);
     const size_t o_first = take(4 * (size_t)((P + 31) / 32));
@@ -1007,6 +1057,10 @@ void build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64_t P,
     a.loff = g->loff;
     a.tasks = g->tasks;
     a.comp = g->comp;
+    a.zrow = g->zrow;
+    a.zbits = g->zbits;
+    a.zowner = g->zowner;
+    a.zcap = g->zcap;
     graph_views(g, &a.view, &a.view_comp);
     a.view_at = g->view;
     a.view_comp_at = g->view_comp;
@@ -1015,11 +1069,12 @@ void build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64_t P,
     a.cta_tasks = tt.cta_unit_tasks;
     a.slice_max = tt.slice_max;
     UnitLists L;
-    auto take_units = [&](int64_t ns, int64_t nl) {
-        L.bytes = sizeof(Unit) * (size_t)std::max<int64_t>(ns + nl, 1);
+    auto take_units = [&](int64_t ns, int64_t nl, int64_t nz) {
+        L.bytes = sizeof(Unit) * (size_t)std::max<int64_t>(ns + nl + nz, 1);
         L.mem = al.get(L.bytes);
         a.large = L.large = static_cast<Unit*>(L.mem);
         a.small = L.small = L.large + nl;
+        a.zone = L.zone = L.small + ns;
         // the graph owns them from here on, whatever fails next
         adopt_units(g, L, tt);
     };
@@ -1028,17 +1083,20 @@ void build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64_t P,
         // for each full unit of tasks; a large pivot has over kSmallMaxOutdeg
         // of the edges, and one slice (d^2 <= 2m)
         static_assert(2 * kBuildOnePairs <= (int64_t)kMaxSlice * kMaxSlice, "one slice a pivot");
-        take_units(std::min(n, P) + P / tt.warp_unit_tasks + 1, P / kSmallMaxOutdeg + P / tt.cta_unit_tasks + 1);
+        take_units(std::min(n, P) + P / tt.warp_unit_tasks + 1, P / kSmallMaxOutdeg + P / tt.cta_unit_tasks + 1,
+                   P / kZoneMinPivot + P / kZoneTasks + 1);
         launch(kPhaseInsert, kPhaseEnd);
         read_tally();
     } else {
         launch(kPhaseGraph, kPhaseUnits);
         read_tally();
-        take_units((int64_t)h.nsmall, (int64_t)h.nlarge);
+        take_units((int64_t)h.nsmall, (int64_t)h.nlarge, (int64_t)h.nzone);
         launch(kPhaseUnits, kPhaseEnd);
     }
     g->n_small = h.nsmall;
     g->n_large = h.nlarge;
+    g->n_zone = h.nzone;
+    g->covered = h.covered;
     g->m = (int64_t)h.m;
     g->n_tasks = (int64_t)h.tasks;
     g->stats.m = g->m;

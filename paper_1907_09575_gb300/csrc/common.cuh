@@ -172,6 +172,15 @@ struct tc_graph {
     uint64_t* tnew = nullptr;   // per-vertex accumulator in new labels, n
     unsigned* tlow = nullptr;   // 32-bit per-task shares (per-vertex counts), n, on demand
     size_t tlow_bytes = 0;
+    // dense zones (zone.cuh); zcap = 0: none
+    int64_t zcap = 0;           // blocks there is room for
+    uint2* zrow = nullptr;      // per row: blocks, first zoned edge
+    uint32_t* zbits = nullptr;
+    uint32_t* zowner = nullptr; // row of a row's first block
+    struct Unit* zone_units = nullptr;
+    int64_t n_zone = 0;
+    uint64_t covered = 0;       // tail entries the zones hold, of pivots that use them
+
     size_t zero_bytes = 0;      // [counters | comp_totals | tnew | tlow (small graphs)] are one range
     bool tlow_in_arena = false;
 
@@ -203,11 +212,13 @@ struct HostCopy {
     int32_t* perm = nullptr;    // n
 };
 
-// A <j,i,k> task: edge (i,j) of U with the part of U_i after j nonempty.
-struct Task {
-    int64_t start;   // index in adj of the first entry of U_i after j
-    int32_t len;     // number of entries of U_i after j (> 0)
+// A <j,i,k> task: edge (i,j) of U with the part of U_i after j nonempty; one
+// 16-byte load.
+struct __align__(16) Task {
+    uint32_t start;  // index in adj of the first entry of U_i after j (m < 2^31)
+    int32_t len;     // entries of U_i after j, those in dense zones aside (>= 0)
     int32_t i;       // row (new label), for per-vertex credit
+    uint32_t zone;   // the row's zone blocks (zone.cuh), 0 when the list holds the whole tail
 };
 
 // A work unit: graph g (index into the view table), pivot j, a slice of U_j
@@ -237,6 +248,9 @@ struct GraphView {
                                   // graph index pivots from their block's start)
     int32_t i0, i1;               // tiles: the rows counted by this launch ...
     int64_t tail_shift;           // ... whose entries start this far into adj
+    const uint2* zrow;            // dense zones (zone.cuh), or null
+    const uint32_t* zbits;
+    const uint32_t* zowner;
 };
 
 // Device counters of one count: queue heads, the total, and work done by the
@@ -249,5 +263,7 @@ enum : int {
     CTR_TASKS = 5,
     CTR_PROBES = 7,
     CTR_STAGED = 9,
+    CTR_ZONE_HEAD = 11,
+    CTR_MID_HEAD = 12,
     CTR_COUNT = 16
 };

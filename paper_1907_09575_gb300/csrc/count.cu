@@ -30,6 +30,7 @@
 
 #include "common.cuh"
 #include "tc_internal.cuh"
+#include "zone.cuh"
 
 namespace tc {
 namespace {
@@ -268,6 +269,51 @@ __device__ __forceinline__ void tag_insert2(unsigned* t2, int k, int q) {
     unsigned* s = t2 + (p >> kTag2Shift);
     if (atomicCAS(s, kTagEmpty, ((unsigned)q << kTag2Shift) | (p & kTag2Mask)) != kTagEmpty) atomicExch(s, kTagMulti);
 }
+
+// The tag table of one warp, for a pivot of at most kMidEntries entries: the
+// same on the 31 bits of a label (labels are below 2^31 - 1, and the -1 of a
+// lane without a probe becomes 2^31 - 1: a miss), which leaves room for the
+// rank beside the longer tags of smaller tables.
+constexpr int kMidEntries = kMidMaxOutdeg;           // 256: ranks of 8 bits
+constexpr int kMidSlotBits = 10, kMidSlots = 1 << kMidSlotBits;
+constexpr int kMidSlot2Bits = 8, kMidSlots2 = 1 << kMidSlot2Bits;
+constexpr int kMidTag = 31 - kMidSlotBits, kMidTag2 = 31 - kMidSlot2Bits;
+static_assert(kMidEntries <= (1 << (31 - kMidTag2)), "ranks fit both tables below bit 31");
+constexpr unsigned kMid31 = 0x7fffffffu;
+
+struct MidTab {
+    const unsigned* t1;
+    const unsigned* t2;
+    const int32_t* row;
+    int dp;
+    __device__ int slow(int k) const {
+        const unsigned p = ((unsigned)k * kTagMul2) & kMid31;
+        const unsigned w = t2[p >> kMidTag2];
+        if (w != kTagMulti)
+            return ((w ^ p) & (0x80000000u | ((1u << kMidTag2) - 1u))) == 0 ? (int)(w >> kMidTag2) : -1;
+        int a = 0, b = dp;
+        while (a < b) {
+            const int c = (a + b) >> 1;
+            if (__ldg(row + c) < k) a = c + 1; else b = c;
+        }
+        return (a < dp && __ldg(row + a) == k) ? a : -1;
+    }
+    template <bool PV>
+    __device__ __forceinline__ int find(int k) const {
+        const unsigned p = ((unsigned)k * kTagMul) & kMid31;
+        const unsigned w = t1[p >> kMidTag];
+        if (w == kTagMulti) return slow(k);
+        return ((w ^ p) & (0x80000000u | ((1u << kMidTag) - 1u))) == 0 ? (int)(w >> kMidTag) : -1;
+    }
+    __device__ __forceinline__ unsigned bit(int k) const { return find<false>(k) >= 0; }
+    __device__ __forceinline__ void probe_credit(int k, unsigned* cnt, unsigned& mine) const {
+        const int r = find<true>(k);
+        mine += r >= 0;
+        add_if(&cnt[r], r >= 0);
+    }
+    __device__ __forceinline__ void credit(unsigned* cnt, int r) const { atomicAdd(&cnt[r], 1u); }
+    __device__ __forceinline__ unsigned credited(const unsigned* cnt, int r) const { return cnt[r]; }
+};
 
 // Search (the list-based joint traversal of Section 3.1, lane-parallel): the
 // sorted pivot row U_j (at most 64 entries) sits in shared memory and each
@@ -983,6 +1029,136 @@ __global__ void __launch_bounds__(256, TC_LARGE_MINB)
     }
 }
 
+// ---------------------------------------------------------------------------
+// Pivots of kZoneMinPivot+1 .. kMidEntries entries, the units of the zone
+// kernel (at most 248 tasks), one warp each.  What the zones leave of such a
+// pivot's tails is little -- at RMAT scale 20 about 15 entries of each of 220
+// tasks -- and a CTA spent more on a unit's chain of loads and barriers (4 us
+// of table building) than on its probes; a warp with a table of its own needs
+// no barrier, and 32 of them on an SM hide one another's loads.  The table is
+// a bitmap (672 words and their rank prefixes) or, for a wider span, 1,024
+// tag slots with 256 more for the entries that share one.
+//
+// Dynamic shared memory of a warp: bases (32 int64) | table (kMidSlots words)
+// | second table (kMidSlots2) | hit counters (PV: kMidEntries).
+// ---------------------------------------------------------------------------
+constexpr int kMidThreads = 256;
+constexpr int kMidBitWords = (kMidSlots * 2 / 3) & ~31;
+constexpr size_t mid_warp_words(bool pv) { return 64 + kMidSlots + kMidSlots2 + (pv ? kMidEntries : 0); }
+
+template <bool PV, class Tab>
+__device__ __forceinline__ void mid_probe(const GraphView& G, const Unit& U, const Tab& T, unsigned* cnt,
+                                          int64_t* s_base, unsigned* tlow, int64_t rb, int dp, uint64_t& hits,
+                                          uint64_t& probes) {
+    const int lane = threadIdx.x & 31;
+    uint64_t uh = 0;
+    for (int64_t tb = U.t0; tb < U.t1; tb += 32)
+        warp_probe_group<PV, false>(G.tasks, tb, U.t1, G.adj, T, cnt, G.tnew, tlow, s_base, U.t0, nullptr, nullptr,
+                                    uh, probes, TaskWindow{0, 0, 0});
+    hits += uh;
+    __syncwarp();
+    if (PV) {
+        for (int r = lane; r < dp; r += 32) {
+            const unsigned h = T.credited(cnt, r);
+            if (h) atomicAdd(&G.tnew[G.adj[rb + r]], (unsigned long long)h);
+        }
+        uh = warp_sum_u64(uh);
+        if (lane == 0 && uh) atomicAdd(&G.tnew[U.j], (unsigned long long)uh);
+    }
+}
+
+template <bool PV>
+__global__ void __launch_bounds__(kMidThreads, 4)
+    k_mid(const GraphView* __restrict__ views, const Unit* __restrict__ units, int64_t nunits, unsigned* tlow,
+          unsigned long long* __restrict__ ctr) {
+    extern __shared__ __align__(16) unsigned smem[];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    unsigned* mine = smem + (size_t)w * mid_warp_words(PV);
+    int64_t* s_base = reinterpret_cast<int64_t*>(mine);
+    unsigned* tab = mine + 64;
+    unsigned* t2 = tab + kMidSlots;
+    unsigned* cnt = t2 + kMidSlots2;
+    GraphAcc acc;
+    uint64_t probes = 0, staged = 0;
+    unsigned long long nu = 0, nt = 0;
+    while (true) {
+        long long u = 0;
+        if (lane == 0) u = (long long)atomicAdd(&ctr[CTR_MID_HEAD], 1ull);
+        u = __shfl_sync(0xffffffffu, u, 0);
+        if (u >= nunits) break;
+        const Unit U = units[u];
+        const GraphView G = views[U.g];
+        const int64_t rb = off_at(G, U.j);
+        const int64_t d = off_at(G, U.j + 1) - rb;
+        if (d > kMidEntries) continue;   // a CTA unit
+        const int dp = (int)d;
+        acc.to(unit_target(G, U));
+        const int lo = G.adj[rb], hi = G.adj[rb + dp - 1];
+        if (PV)
+            for (int q = lane; q < dp; q += 32) cnt[q] = 0;
+        if ((int64_t)hi - lo + 1 < 32ll * kMidBitWords) {   // labels + guard bit
+            const int words = ((hi - lo + 1) >> 5) + 1;
+            for (int q = lane; q < words; q += 32) tab[q] = 0;
+            __syncwarp();
+            for (int q = lane; q < dp; q += 32) {
+                const int k = G.adj[rb + q] - lo;
+                atomicOr(&tab[k >> 5], 1u << (k & 31));
+            }
+            __syncwarp();
+            unsigned short* pre = reinterpret_cast<unsigned short*>(tab + kMidBitWords);
+            if (PV) {
+                int before = 0;   // prefix popcounts, 32 words at a time
+                for (int q0 = 0; q0 < words; q0 += 32) {
+                    const int c = q0 + lane < words ? __popc(tab[q0 + lane]) : 0;
+                    const int inc = warp_incl_scan_i32(c);
+                    if (q0 + lane < words) pre[q0 + lane] = (unsigned short)(before + inc - c);
+                    before += __shfl_sync(0xffffffffu, inc, 31);
+                }
+                __syncwarp();
+            }
+            const BitTab T{tab, pre, lo, hi};
+            mid_probe<PV>(G, U, T, cnt, s_base, tlow, rb, dp, acc.hits, probes);
+        } else {
+            for (int q = lane; q < kMidSlots + kMidSlots2; q += 32) tab[q] = kTagEmpty;
+            __syncwarp();
+            for (int q = lane; q < dp; q += 32) {
+                const int k = G.adj[rb + q];
+                const unsigned p = ((unsigned)k * kTagMul) & kMid31;
+                unsigned* slot = tab + (p >> kMidTag);
+                const unsigned word = ((unsigned)q << kMidTag) | (p & ((1u << kMidTag) - 1u));
+                if (atomicCAS(slot, kTagEmpty, word) != kTagEmpty) {
+                    // a shared slot: this entry and the one displaced (if
+                    // still there) move to the second table
+                    const unsigned old = atomicExch(slot, kTagMulti);
+                    for (int h = 0; h < 2; ++h) {
+                        if (h == 1 && old == kTagMulti) break;
+                        const int qq = h == 0 ? q : (int)(old >> kMidTag);
+                        const unsigned p2 = ((unsigned)G.adj[rb + qq] * kTagMul2) & kMid31;
+                        unsigned* s2 = t2 + (p2 >> kMidTag2);
+                        if (atomicCAS(s2, kTagEmpty, ((unsigned)qq << kMidTag2) | (p2 & ((1u << kMidTag2) - 1u))) !=
+                            kTagEmpty)
+                            atomicExch(s2, kTagMulti);
+                    }
+                }
+            }
+            __syncwarp();
+            const MidTab T{tab, t2, G.adj + rb, dp};
+            mid_probe<PV>(G, U, T, cnt, s_base, tlow, rb, dp, acc.hits, probes);
+        }
+        staged += (uint64_t)dp;
+        nu += 1;
+        nt += (unsigned long long)(U.t1 - U.t0);
+        __syncwarp();   // the table is rebuilt by the next unit
+    }
+    acc.flush();
+    if (lane == 0 && nu) {
+        atomicAdd(&ctr[CTR_UNITS + 1], nu);
+        atomicAdd(&ctr[CTR_TASKS + 1], nt);
+        atomicAdd(&ctr[CTR_PROBES + 1], (unsigned long long)probes);
+        atomicAdd(&ctr[CTR_STAGED + 1], (unsigned long long)staged);
+    }
+}
+
 // per-vertex counts in original ids: the 64-bit accumulator plus, when used,
 // the 32-bit per-task shares
 __global__ void k_gather_pv(const unsigned long long* __restrict__ tnew, const unsigned* __restrict__ tlow,
@@ -1015,8 +1191,8 @@ __device__ __forceinline__ int find_graph(const int64_t* __restrict__ vpre, int 
 }
 
 __global__ void k_unit_counts(const GraphView* __restrict__ views, const int64_t* __restrict__ vpre,
-                              int num, int64_t V, int small_max, int tw, int tcta, int slice,
-                              int32_t* __restrict__ cs, int32_t* __restrict__ cl) {
+                              int num, int64_t V, int small_max, int mid_max, int tw, int tcta, int slice,
+                              int32_t* __restrict__ cs, int32_t* __restrict__ cl, int32_t* __restrict__ cz) {
     for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < V;
          x += (int64_t)gridDim.x * blockDim.x) {
         const int64_t v = V - 1 - x;
@@ -1026,10 +1202,11 @@ __global__ void k_unit_counts(const GraphView* __restrict__ views, const int64_t
         const int64_t dp = off_at(G, j + 1) - off_at(G, j);
         const int64_t nt = G.loff[j + 1] - G.loff[j];
         int32_t a = 0, b = 0;
+        cz[x] = G.zrow && dp > kZoneMinPivot ? (int32_t)((nt + kZoneTasks - 1) / kZoneTasks) : 0;
         if (dp > 0 && nt > 0) {
             if (dp <= small_max) {
                 a = (int32_t)((nt + tw - 1) / tw);
-            } else {
+            } else if (!(G.zrow && dp > kZoneMinPivot && dp <= mid_max)) {
                 const int64_t slices = (dp + slice - 1) / slice;
                 b = (int32_t)(slices * ((nt + tcta - 1) / tcta));
             }
@@ -1040,9 +1217,10 @@ __global__ void k_unit_counts(const GraphView* __restrict__ views, const int64_t
 }
 
 __global__ void k_unit_fill(const GraphView* __restrict__ views, const int64_t* __restrict__ vpre,
-                            int num, int64_t V, int small_max, int tw, int tcta, int slice,
+                            int num, int64_t V, int small_max, int mid_max, int tw, int tcta, int slice,
                             const int64_t* __restrict__ ps, const int64_t* __restrict__ pl,
-                            Unit* __restrict__ us, Unit* __restrict__ ul) {
+                            const int64_t* __restrict__ pz, Unit* __restrict__ us, Unit* __restrict__ ul,
+                            Unit* __restrict__ uz) {
     for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < V;
          x += (int64_t)gridDim.x * blockDim.x) {
         const int64_t v = V - 1 - x;
@@ -1052,11 +1230,16 @@ __global__ void k_unit_fill(const GraphView* __restrict__ views, const int64_t* 
         const int64_t dp = off_at(G, j + 1) - off_at(G, j);
         const int64_t a = G.loff[j], b = G.loff[j + 1];
         if (dp <= 0 || b <= a) continue;
+        if (G.zrow && dp > kZoneMinPivot) {
+            int64_t p = pz[x];
+            for (int64_t t = a; t < b; t += kZoneTasks)
+                uz[p++] = Unit{(int32_t)j, 0, g, 0, t, min64(t + kZoneTasks, b)};
+        }
         if (dp <= small_max) {
             int64_t p = ps[x];
             for (int64_t t = a; t < b; t += tw)
                 us[p++] = Unit{(int32_t)j, 0, g, 0, t, min64(t + tw, b)};
-        } else {
+        } else if (!(G.zrow && dp > kZoneMinPivot && dp <= mid_max)) {
             const int64_t slices = (dp + slice - 1) / slice;
             int64_t p = pl[x];
             for (int64_t t = a; t < b; t += tcta)
@@ -1084,42 +1267,49 @@ void plan_units(UnitPlan& P, const GraphView* views_dev, const int64_t* vpre_dev
     P.t = t;
     P.cs = Buf<int32_t>(al, (size_t)std::max<int64_t>(V, 1));
     P.cl = Buf<int32_t>(al, (size_t)std::max<int64_t>(V, 1));
+    P.cz = Buf<int32_t>(al, (size_t)std::max<int64_t>(V, 1));
     P.ps = Buf<int64_t>(al, (size_t)(V + 1));
     P.pl = Buf<int64_t>(al, (size_t)(V + 1));
+    P.pz = Buf<int64_t>(al, (size_t)(V + 1));
     if (V > 0) {
         Prof prof_("k_unit_counts", st);
         k_unit_counts<<<grid_for(V, 256, G), 256, 0, st>>>(views_dev, vpre_dev, num, V,
-                                                           t.small_max_outdeg, t.warp_unit_tasks,
+                                                           t.small_max_outdeg, mid_max_outdeg(t), t.warp_unit_tasks,
                                                            t.cta_unit_tasks, t.slice_max, P.cs.get(),
-                                                           P.cl.get());
+                                                           P.cl.get(), P.cz.get());
     }
     TC_LAUNCH_CHECK();
     exclusive_scan2_i32_to_i64(P.cs.get(), P.ps.get(), P.ps.get() + V, P.cl.get(), P.pl.get(), P.pl.get() + V, V,
                                al, st);
+    exclusive_scan_i32_to_i64(P.cz.get(), P.pz.get(), V, P.pz.get() + V, al, st);
 }
 
-UnitLists fill_units(UnitPlan& P, int64_t ns, int64_t nl, Alloc& al, cudaStream_t st) {
+UnitLists fill_units(UnitPlan& P, int64_t ns, int64_t nl, int64_t nz, Alloc& al, cudaStream_t st) {
     const unsigned G = (unsigned)(num_sms() * 8);
     UnitLists L;
-    L.bytes = sizeof(Unit) * (size_t)std::max<int64_t>(ns + nl, 1);
+    L.bytes = sizeof(Unit) * (size_t)std::max<int64_t>(ns + nl + nz, 1);
     L.mem = al.get(L.bytes);
     L.large = static_cast<Unit*>(L.mem);
     L.small = L.large + nl;
+    L.zone = L.small + ns;
     L.nlarge = nl;
     L.nsmall = ns;
+    L.nzone = nz;
     if (P.V > 0) {
         {
             Prof prof_("k_unit_fill", st);
             k_unit_fill<<<grid_for(P.V, 256, G), 256, 0, st>>>(
-                P.views, P.vpre, P.num, P.V, P.t.small_max_outdeg, P.t.warp_unit_tasks,
-                P.t.cta_unit_tasks, P.t.slice_max, P.ps.get(), P.pl.get(), L.small, L.large);
+                P.views, P.vpre, P.num, P.V, P.t.small_max_outdeg, mid_max_outdeg(P.t), P.t.warp_unit_tasks,
+                P.t.cta_unit_tasks, P.t.slice_max, P.ps.get(), P.pl.get(), P.pz.get(), L.small, L.large, L.zone);
         }
         TC_LAUNCH_CHECK();
     }
     P.cs.release();
     P.cl.release();
+    P.cz.release();
     P.ps.release();
     P.pl.release();
+    P.pz.release();
     return L;
 }
 
@@ -1127,11 +1317,12 @@ UnitLists build_unit_lists(const GraphView* views_dev, const int64_t* vpre_dev, 
                            const tc_tuning& t, Alloc& al, cudaStream_t st) {
     UnitPlan P;
     plan_units(P, views_dev, vpre_dev, num, V, t, al, st);
-    int64_t ns = 0, nl = 0;
+    int64_t ns = 0, nl = 0, nz = 0;
     TC_CUDA(cudaMemcpyAsync(&ns, P.ps.get() + V, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+    TC_CUDA(cudaMemcpyAsync(&nz, P.pz.get() + V, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     TC_CUDA(cudaMemcpyAsync(&nl, P.pl.get() + V, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     TC_CUDA(cudaStreamSynchronize(st));
-    return fill_units(P, ns, nl, al, st);
+    return fill_units(P, ns, nl, nz, al, st);
 }
 
 void adopt_units(tc_graph* g, const UnitLists& L, const tc_tuning& tt) {
@@ -1140,11 +1331,24 @@ void adopt_units(tc_graph* g, const UnitLists& L, const tc_tuning& tt) {
     g->units_bytes = L.bytes;
     g->small_units = L.small;
     g->large_units = L.large;
+    g->zone_units = L.zone;
+    g->n_zone = L.nzone;
     g->n_small = L.nsmall;
     g->n_large = L.nlarge;
     g->units_tuning = tt;
     g->stats.small_units = L.nsmall;
     g->stats.large_units = L.nlarge;
+}
+
+UnitLists units_of(const tc_graph* g) {
+    UnitLists L;
+    L.large = g->large_units;
+    L.small = g->small_units;
+    L.zone = g->zone_units;
+    L.nlarge = g->n_large;
+    L.nsmall = g->n_small;
+    L.nzone = g->n_zone;
+    return L;
 }
 
 size_t count_smem_bytes(bool pv, int threads, int unit_tasks) {
@@ -1211,6 +1415,32 @@ void launch_count(const GraphView* views_dev, const UnitLists& L, const tc_tunin
     }
 }
 
+void launch_mid(const GraphView* views_dev, const UnitLists& L, const tc_tuning& t, bool pv,
+                unsigned long long* ctr, cudaStream_t st, unsigned* tlow, bool profile) {
+    if (L.nzone == 0 || mid_max_outdeg(t) == 0) return;
+    const size_t smem = sizeof(unsigned) * mid_warp_words(pv) * (kMidThreads / 32);
+    const unsigned blocks = (unsigned)std::min<int64_t>((L.nzone + kMidThreads / 32 - 1) / (kMidThreads / 32),
+                                                        (int64_t)num_sms() * 4);
+    auto go = [&]() {
+        if (pv) k_mid<true><<<blocks, kMidThreads, smem, st>>>(views_dev, L.zone, L.nzone, tlow, ctr);
+        else k_mid<false><<<blocks, kMidThreads, smem, st>>>(views_dev, L.zone, L.nzone, tlow, ctr);
+    };
+    if (profile) {
+        Prof prof_("k_mid", st);
+        go();
+    } else {
+        go();
+    }
+    TC_LAUNCH_CHECK();
+}
+
+void prepare_mid() {
+    TC_CUDA(cudaFuncSetAttribute(k_mid<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(sizeof(unsigned) * mid_warp_words(true) * (kMidThreads / 32))));
+    TC_CUDA(cudaFuncSetAttribute(k_mid<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(sizeof(unsigned) * mid_warp_words(false) * (kMidThreads / 32))));
+}
+
 void build_units(tc_graph* g, const tc_tuning& t, cudaStream_t st) {
     const tc_tuning tt = clamp_tuning(t);
     Alloc& al = g->alloc;
@@ -1229,12 +1459,11 @@ void count_components(tc_graph* g, const tc_tuning& t, uint64_t* comp_totals_dev
     TC_CUDA(cudaMemsetAsync(g->counters, 0,
                             (size_t)(reinterpret_cast<char*>(g->comp_totals + g->num_comps) -
                                      reinterpret_cast<char*>(g->counters)), st));
-    UnitLists L;
-    L.large = g->large_units;
-    L.small = g->small_units;
-    L.nlarge = g->n_large;
-    L.nsmall = g->n_small;
+    const UnitLists L = units_of(g);
     launch_count(g->view_comp, L, tt, false, g->counters, st, true, nullptr);
+    if (L.nzone > 0) prepare_mid();
+    launch_mid(g->view_comp, L, tt, false, g->counters, st, nullptr, true);
+    launch_zone(g->view_comp, L, false, g->counters, st, nullptr, true);
     TC_CUDA(cudaMemcpyAsync(comp_totals_dev, g->comp_totals, sizeof(uint64_t) * (size_t)g->num_comps,
                             cudaMemcpyDeviceToDevice, st));
 }
@@ -1257,12 +1486,11 @@ void count(tc_graph* g, const tc_tuning& t, uint64_t* total_dev, uint64_t* per_v
         }
         TC_CUDA(cudaMemsetAsync(g->tlow, 0, g->tlow_bytes, st));
     }
-    UnitLists L;
-    L.large = g->large_units;
-    L.small = g->small_units;
-    L.nlarge = g->n_large;
-    L.nsmall = g->n_small;
+    const UnitLists L = units_of(g);
     launch_count(g->view, L, tt, pv, g->counters, st, true, tlow32 ? g->tlow : nullptr);
+    if (L.nzone > 0) prepare_mid();
+    launch_mid(g->view, L, tt, pv, g->counters, st, tlow32 ? g->tlow : nullptr, true);
+    launch_zone(g->view, L, pv, g->counters, st, tlow32 ? g->tlow : nullptr, true);
     if (pv && g->n > 0) {
         {
             Prof prof_("k_gather_pv", st);

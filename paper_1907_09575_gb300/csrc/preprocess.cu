@@ -23,6 +23,7 @@
 
 #include "common.cuh"
 #include "tc_internal.cuh"
+#include "zone.cuh"
 
 namespace tc {
 namespace {
@@ -504,15 +505,30 @@ __global__ void k_task_count_last(const OffT* __restrict__ off, const int32_t* _
 #endif
 constexpr int kFillILP = TC_FILL_ILP;
 
+constexpr unsigned long long kBigPivot = 1ull << 63;   // in fill[j]: the pivot takes part in the zones
+
+template <class OffT>
+__global__ void k_fill_init(const OffT* __restrict__ off, const int64_t* __restrict__ loff, int64_t n,
+                            unsigned long long* __restrict__ fill) {
+    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
+         v += (int64_t)gridDim.x * blockDim.x)
+        fill[v] = (unsigned long long)loff[v] |
+                  ((int64_t)off[v + 1] - (int64_t)off[v] > kZoneMinPivot ? kBigPivot : 0ull);
+}
+
+// zrow: the dense zones (zone.cuh), or null; covered += the entries
+// they take from the lists
 template <class OffT>
 __global__ void k_task_fill(const uint64_t* __restrict__ keys, int64_t m, int bits,
                             const OffT* __restrict__ off, unsigned long long* __restrict__ fill,
-                            Task* __restrict__ tasks) {
+                            Task* __restrict__ tasks, const uint2* __restrict__ zrow, unsigned long long* __restrict__ covered) {
     const uint64_t mask = (1ull << bits) - 1ull;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    unsigned long long cut = 0;
     for (int64_t e0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e0 < m; e0 += stride * kFillILP) {
         int64_t i[kFillILP], len[kFillILP];
         int32_t j[kFillILP];
+        uint2 zr[kFillILP];
 #pragma unroll
         for (int u = 0; u < kFillILP; ++u) {
             const int64_t e = e0 + u * stride;
@@ -522,6 +538,7 @@ __global__ void k_task_fill(const uint64_t* __restrict__ keys, int64_t m, int bi
                 i[u] = (int64_t)(k >> bits);
                 j[u] = (int32_t)(k & mask);
                 len[u] = (int64_t)off[i[u] + 1] - e - 1;
+                zr[u] = zrow ? zrow[i[u]] : make_uint2(0, 0);
             }
         }
         unsigned long long slot[kFillILP];
@@ -531,13 +548,18 @@ __global__ void k_task_fill(const uint64_t* __restrict__ keys, int64_t m, int bi
 #pragma unroll
         for (int u = 0; u < kFillILP; ++u)
             if (len[u] > 0) {
+                const int64_t e = e0 + u * stride;
                 Task t;
-                t.start = e0 + u * stride + 1;
-                t.len = (int32_t)len[u];
+                t.start = (uint32_t)(e + 1);
+                t.len = zone_cut(zr[u], (slot[u] & kBigPivot) != 0, e, (int)len[u], &t.zone);
                 t.i = (int32_t)i[u];
-                tasks[slot[u]] = t;
+                cut += (unsigned long long)(len[u] - t.len);
+                tasks[slot[u] & ~kBigPivot] = t;
             }
     }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) cut += __shfl_xor_sync(0xffffffffu, cut, o);
+    if ((threadIdx.x & 31) == 0 && cut) atomicAdd(covered, cut);
 }
 
 template <class OffT>
@@ -636,6 +658,9 @@ void graph_arena(tc_graph* g, int64_t cap_m, bool off64, int32_t num_comps) {
     const size_t o_off = take((off64 ? 8 : 4) * (n + 1)), o_adj = take(4 * m), o_perm = take(4 * nv);
     const size_t o_loff = take(8 * (n + 1)), o_tasks = take(sizeof(Task) * m);
     const size_t o_view = take(sizeof(GraphView)), o_vc = take(sizeof(GraphView));
+    const int64_t zcap = zone_capacity(cap_m);
+    const size_t o_zrow = take(zcap ? 8 * nv : 0);
+    const size_t o_zbits = take(4 * (size_t)kZoneWords * (size_t)zcap), o_zown = take(4 * (size_t)zcap);
     const size_t o_comp = take(num_comps > 0 ? 4 * nv : 0);
     const size_t o_ctr = take(sizeof(unsigned long long) * CTR_COUNT);
     const size_t o_ctot = take(8 * (size_t)std::max(num_comps, 0));
@@ -654,6 +679,12 @@ void graph_arena(tc_graph* g, int64_t cap_m, bool off64, int32_t num_comps) {
     g->counters = reinterpret_cast<unsigned long long*>(a + o_ctr);
     g->tnew = reinterpret_cast<uint64_t*>(a + o_tnew);
     g->zero_bytes = need - o_ctr;
+    g->zcap = zcap;
+    if (zcap > 0) {
+        g->zrow = reinterpret_cast<uint2*>(a + o_zrow);
+        g->zbits = reinterpret_cast<uint32_t*>(a + o_zbits);
+        g->zowner = reinterpret_cast<uint32_t*>(a + o_zown);
+    }
     if (low) {
         g->tlow = reinterpret_cast<unsigned*>(a + o_tlow);
         g->tlow_in_arena = true;
@@ -675,6 +706,9 @@ void graph_views(const tc_graph* g, GraphView* v, GraphView* vc) {
     v->total = g->counters + CTR_TOTAL;
     v->n = g->n;
     v->off64 = g->off64 ? 1 : 0;
+    v->zrow = g->zrow;
+    v->zbits = g->zbits;
+    v->zowner = g->zowner;
     *vc = *v;
     vc->tnew = nullptr;
     vc->comp = g->comp;
@@ -1011,8 +1045,8 @@ void preprocess_with_components(tc_graph* g, const int32_t* src_in, const int32_
     }
 
     // a6 tasks grouped by pivot j
-    Buf<unsigned long long> probes(al, 2);   // [0] <j,i,k> probes, [1] <i,j,k> probes
-    TC_CUDA(cudaMemsetAsync(probes.get(), 0, 2 * sizeof(unsigned long long), st));
+    Buf<unsigned long long> probes(al, 3);   // [0] <j,i,k> probes, [1] <i,j,k> probes, [2] entries in zones
+    TC_CUDA(cudaMemsetAsync(probes.get(), 0, 3 * sizeof(unsigned long long), st));
     int32_t* tcount = dplus.get();  // reuse
     if (n > 0) {
         {
@@ -1040,16 +1074,27 @@ void preprocess_with_components(tc_graph* g, const int32_t* src_in, const int32_
     exclusive_scan_i32_to_i64(tcount, g->loff, n, g->loff + n, al, st);
     if (m > 0) {
         Buf<unsigned long long> fill(al, (size_t)std::max<int64_t>(n, 1));
-        TC_CUDA(cudaMemcpyAsync(fill.get(), g->loff, sizeof(int64_t) * (size_t)std::max<int64_t>(n, 1),
-                                cudaMemcpyDeviceToDevice, st));
+        if (g->zcap > 0) zone_rows(g, reinterpret_cast<unsigned*>(scal.get() + 5), st);
+        {
+            Prof prof_("k_fill_init", st);
+            if (g->off64)
+                k_fill_init<int64_t><<<grid_for(n, kT, G), kT, 0, st>>>(static_cast<const int64_t*>(g->off), g->loff,
+                                                                        n, fill.get());
+            else
+                k_fill_init<int32_t><<<grid_for(n, kT, G), kT, 0, st>>>(static_cast<const int32_t*>(g->off), g->loff,
+                                                                        n, fill.get());
+        }
+        TC_LAUNCH_CHECK();
         {
             Prof prof_("k_task_fill", st);
             if (g->off64)
                 k_task_fill<int64_t><<<grid_for(m, kT, G), kT, 0, st>>>(
-                    keys, m, bits, static_cast<const int64_t*>(g->off), fill.get(), g->tasks);
+                    keys, m, bits, static_cast<const int64_t*>(g->off), fill.get(), g->tasks, g->zrow,
+                    probes.get() + 2);
             else
                 k_task_fill<int32_t><<<grid_for(m, kT, G), kT, 0, st>>>(
-                    keys, m, bits, static_cast<const int32_t*>(g->off), fill.get(), g->tasks);
+                    keys, m, bits, static_cast<const int32_t*>(g->off), fill.get(), g->tasks, g->zrow,
+                    probes.get() + 2);
         }
         TC_LAUNCH_CHECK();
     }
@@ -1087,8 +1132,8 @@ void preprocess_with_components(tc_graph* g, const int32_t* src_in, const int32_
     TC_CUDA(cudaMemcpyAsync(gvpre.get(), hv, sizeof(hv), cudaMemcpyHostToDevice, st));
     UnitPlan plan;
     plan_units(plan, g->view, gvpre.get(), 1, n, def, al, st);
-    unsigned long long hprobes[2] = {0, 0};
-    int64_t ntasks = 0, ns = 0, nl = 0;
+    unsigned long long hprobes[3] = {0, 0, 0};
+    int64_t ntasks = 0, ns = 0, nl = 0, nz = 0;
     int herr = 0;
     TC_CUDA(cudaMemcpyAsync(&maxout, scal.get() + 2, sizeof(int), cudaMemcpyDeviceToHost, st));
     TC_CUDA(cudaMemcpyAsync(&herr, scal.get(), sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -1096,6 +1141,7 @@ void preprocess_with_components(tc_graph* g, const int32_t* src_in, const int32_
     TC_CUDA(cudaMemcpyAsync(&ntasks, g->loff + n, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     TC_CUDA(cudaMemcpyAsync(&ns, plan.ps.get() + n, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     TC_CUDA(cudaMemcpyAsync(&nl, plan.pl.get() + n, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+    TC_CUDA(cudaMemcpyAsync(&nz, plan.pz.get() + n, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     TC_CUDA(cudaStreamSynchronize(st));
     if (herr & 4) TC_FAIL(TC_ETIMEOUT, "tc_preprocess: a sort look-back wait ran past its bound");
     if (herr & 8) TC_FAIL(TC_EUNSUPPORTED, "tc_preprocess: a row of U exceeds the row sort's bound");
@@ -1105,7 +1151,8 @@ void preprocess_with_components(tc_graph* g, const int32_t* src_in, const int32_
     g->stats.probes = hprobes[0];
     g->stats.probes_ijk = hprobes[1];
     g->stats.offset_bytes = (int32_t)ob;
-    UnitLists L = fill_units(plan, ns, nl, al, st);
+    g->covered = hprobes[2];
+    UnitLists L = fill_units(plan, ns, nl, nz, al, st);
     adopt_units(g, L, def);
     g->stats.device_bytes = (int64_t)(g->arena_bytes + g->units_bytes);
 }

@@ -6,6 +6,7 @@ namespace tc {
 
 constexpr int kSmallTable = 128;     // hash slots of a warp unit's table
 constexpr int kSmallMaxOutdeg = 64;  // largest pivot row a warp unit takes
+constexpr int kMidMaxOutdeg = 256;   // largest pivot row counted by one warp, beside the zones
 constexpr int kMaxSlice = 4096;      // largest pivot slice a CTA unit tables
 constexpr int kMaxUnitTasks = 8192;  // 16-bit hit counters; a shared long-task queue
 
@@ -57,15 +58,16 @@ struct UnitLists {
     size_t bytes = 0;
     Unit* large = nullptr;
     Unit* small = nullptr;
-    int64_t nlarge = 0, nsmall = 0;
+    Unit* zone = nullptr;
+    int64_t nlarge = 0, nsmall = 0, nzone = 0;
 };
 
 // Unit building in two phases: plan_units launches the counting kernels and
-// scans (the list sizes land at ps[V], pl[V] on the device); once the host
+// scans (the list sizes land at ps[V], pl[V], pz[V] on the device); once the host
 // knows them, fill_units allocates and fills the lists.
 struct UnitPlan {
-    Buf<int32_t> cs, cl;
-    Buf<int64_t> ps, pl;
+    Buf<int32_t> cs, cl, cz;
+    Buf<int64_t> ps, pl, pz;
     int64_t V = 0;
     int num = 0;
     const GraphView* views = nullptr;
@@ -74,7 +76,8 @@ struct UnitPlan {
 };
 void plan_units(UnitPlan& P, const GraphView* views_dev, const int64_t* vpre_dev, int num, int64_t V,
                 const tc_tuning& t, Alloc& al, cudaStream_t st);
-UnitLists fill_units(UnitPlan& P, int64_t ns, int64_t nl, Alloc& al, cudaStream_t st);
+UnitLists fill_units(UnitPlan& P, int64_t ns, int64_t nl, int64_t nz, Alloc& al, cudaStream_t st);
+UnitLists units_of(const tc_graph* g);
 void adopt_units(tc_graph* g, const UnitLists& L, const tc_tuning& tt);
 
 tc_tuning clamp_tuning(const tc_tuning& t);
@@ -104,6 +107,17 @@ void launch_count_raw(const CountLaunch& c, const GraphView* views_dev, const Un
 void launch_count(const GraphView* views_dev, const UnitLists& L, const tc_tuning& t, bool pv,
                   unsigned long long* ctr, cudaStream_t st, bool profile, unsigned* tlow = nullptr,
                   bool win = false);
+// The pivots that warps count beside the zones (none with buckets everywhere)
+inline int mid_max_outdeg(const tc_tuning& t) { return t.table_mode == 1 ? 0 : kMidMaxOutdeg; }
+void prepare_mid();   // shared-memory attributes: call it outside stream capture
+void launch_mid(const GraphView* views_dev, const UnitLists& L, const tc_tuning& t, bool pv,
+                unsigned long long* ctr, cudaStream_t st, unsigned* tlow, bool profile);
+// Dense zones (zone.cu): the blocks of every row; the zone units' part of a
+// count; the tasks' tails whole again.
+void zone_rows(const tc_graph* g, unsigned* nblocks, cudaStream_t st);
+void launch_zone(const GraphView* views_dev, const UnitLists& L, bool pv, unsigned long long* ctr,
+                 cudaStream_t st, unsigned* tlow, bool profile);
+void zone_restore(const tc_graph* g, cudaStream_t st);
 void build_units(tc_graph* g, const tc_tuning& t, cudaStream_t st);
 void count(tc_graph* g, const tc_tuning& t, uint64_t* total_dev, uint64_t* per_vertex_dev,
            cudaStream_t st);

@@ -86,6 +86,7 @@ void graph_offload(tc_graph* g, cudaStream_t st) {
     const int64_t n = g->n, m = g->m, T = g->n_tasks;
     const size_t ob = g->off64 ? 8 : 4;
     try {
+        zone_restore(g, st);
         take(&h->off, ob * (size_t)(n + 1));
         take(reinterpret_cast<void**>(&h->adj), 4 * (size_t)m);
         take(reinterpret_cast<void**>(&h->loff), 8 * (size_t)(n + 1));
@@ -118,8 +119,12 @@ void graph_offload(tc_graph* g, cudaStream_t st) {
     g->counters = nullptr;
     g->view = g->view_comp = nullptr;
     g->tnew = nullptr;
-    g->small_units = g->large_units = nullptr;
-    g->n_small = g->n_large = 0;
+    g->small_units = g->large_units = g->zone_units = nullptr;
+    g->n_small = g->n_large = g->n_zone = 0;
+    g->zbits = g->zowner = nullptr;
+    g->zrow = nullptr;
+    g->zcap = 0;
+    g->covered = 0;
     g->units_bytes = g->arena_bytes = g->tlow_bytes = 0;
     g->units_tuning = tc_tuning{};
     g->host = h;
@@ -288,7 +293,7 @@ void count_tiled(const tc_graph* g, int64_t budget, Alloc& al, const tc_tuning& 
         TC_CUDA(cudaMemcpyAsync(&cnt[0], P.ps.get() + nJ, 8, cudaMemcpyDeviceToHost, st));
         TC_CUDA(cudaMemcpyAsync(&cnt[1], P.pl.get() + nJ, 8, cudaMemcpyDeviceToHost, st));
         TC_CUDA(cudaStreamSynchronize(st));
-        UnitLists L = fill_units(P, cnt[0], cnt[1], al, st);
+        UnitLists L = fill_units(P, cnt[0], cnt[1], 0, al, st);
         const CountLaunch launch = prepare_count(L, tt, pv, true);
         try {
             for (size_t a = 0; a < need.size(); ++a) {
