@@ -6,6 +6,8 @@
 // a, a+b, a+b+c thresholds, a seeded bijective scramble x -> ((x*A mod 2^s)
 // xor B) * C mod 2^s, and rejection of ids >= n (64 attempts, then the
 // self-loop (0,0)).  Equal output for equal (seed, scale, n, pair index).
+#include <algorithm>
+
 #include "common.cuh"
 #include "tc_internal.cuh"
 
@@ -27,77 +29,96 @@ __host__ __device__ __forceinline__ uint64_t draw(uint64_t key, uint64_t ctr) {
     return mix64(key + (ctr + 1ull) * kGamma);
 }
 
-__global__ void k_rmat(uint64_t key, int scale, uint64_t n, int64_t e0, int64_t count,
-                       uint32_t t1, uint32_t t2, uint32_t t3, uint64_t A, uint64_t B, uint64_t C,
-                       int32_t* __restrict__ src, int32_t* __restrict__ dst) {
-    const uint64_t mask = (1ull << scale) - 1ull;
-    const uint64_t hpa = (uint64_t)((scale + 1) / 2);
+// One attempt at pair e: the two scrambled ids (below 2^scale <= 2^31, so all
+// but the draws is 32-bit arithmetic); false when one of them is >= n.
+struct RmatShape {
+    uint64_t key;
+    uint32_t A, B, C, n, t1, t2, t3;
+    int scale;
+};
+
+__device__ __forceinline__ bool rmat_attempt(const RmatShape& J, uint64_t e, int attempt, uint32_t& u, uint32_t& v) {
+    const uint32_t mask = (1u << J.scale) - 1u;
+    uint64_t z = J.key + ((e * kAttempts + (uint64_t)attempt) * (uint64_t)((J.scale + 1) / 2) + 1ull) * kGamma;
+    u = v = 0;
+    for (int l = 0; l < J.scale; l += 2) {
+        const uint64_t h = mix64(z);
+        z += kGamma;
+        const uint32_t r0 = (uint32_t)h, r1 = (uint32_t)(h >> 32);
+        u = 2 * u + (r0 >= J.t2);
+        v = 2 * v + ((r0 >= J.t1 && r0 < J.t2) || r0 >= J.t3);
+        if (l + 1 < J.scale) {
+            u = 2 * u + (r1 >= J.t2);
+            v = 2 * v + ((r1 >= J.t1 && r1 < J.t2) || r1 >= J.t3);
+        }
+    }
+    u = ((((u * J.A) & mask) ^ J.B) * J.C) & mask;
+    v = ((((v * J.A) & mask) ^ J.B) * J.C) & mask;
+    return u < J.n && v < J.n;
+}
+
+__global__ void k_rmat(RmatShape J, int64_t e0, int64_t count, int32_t* __restrict__ src, int32_t* __restrict__ dst) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count;
          i += (int64_t)gridDim.x * blockDim.x) {
-        const uint64_t e = (uint64_t)(e0 + i);
-        int32_t su = 0, sv = 0;
-        for (int a = 0; a < kAttempts; ++a) {
-            const uint64_t base = (e * kAttempts + (uint64_t)a) * hpa;
-            uint64_t u = 0, v = 0, h = 0;
-            for (int l = 0; l < scale; ++l) {
-                if ((l & 1) == 0) h = draw(key, base + (uint64_t)(l >> 1));
-                const uint32_t r = (l & 1) ? (uint32_t)(h >> 32) : (uint32_t)h;
-                const uint64_t bu = (r >= t2) ? 1ull : 0ull;
-                const uint64_t bv = (r >= t1 && r < t2) || (r >= t3) ? 1ull : 0ull;
-                u = (u << 1) | bu;
-                v = (v << 1) | bv;
-            }
-            u = ((((u * A) & mask) ^ B) * C) & mask;
-            v = ((((v * A) & mask) ^ B) * C) & mask;
-            if (u < n && v < n) {
-                su = (int32_t)u;
-                sv = (int32_t)v;
-                break;
-            }
-        }
-        src[i] = su;
-        dst[i] = sv;
+        uint32_t u = 0, v = 0;
+        int a = 0;
+        while (a < kAttempts && !rmat_attempt(J, (uint64_t)(e0 + i), a, u, v)) ++a;
+        src[i] = a < kAttempts ? (int32_t)u : 0;
+        dst[i] = a < kAttempts ? (int32_t)v : 0;
     }
 }
 
 // Many RMAT requests at once: pair x of the concatenation belongs to the
 // request r with ppre[r] <= x < ppre[r+1]; its ids are offset by vpre[r].
-__global__ void k_rmat_multi(const RmatJob* __restrict__ jobs, const int64_t* __restrict__ ppre,
-                             int nreq, int64_t total, int32_t* __restrict__ src,
-                             int32_t* __restrict__ dst) {
-    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < total;
-         x += (int64_t)gridDim.x * blockDim.x) {
-        int lo = 0, hi = nreq - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (ppre[mid] <= x) lo = mid; else hi = mid - 1;
-        }
-        const RmatJob& J = jobs[lo];
-        const uint64_t e = (uint64_t)(x - ppre[lo]);
-        const uint64_t mask = (1ull << J.scale) - 1ull;
-        const uint64_t hpa = (uint64_t)((J.scale + 1) / 2);
-        int64_t su = 0, sv = 0;
-        for (int a = 0; a < kAttempts; ++a) {
-            const uint64_t base = (e * kAttempts + (uint64_t)a) * hpa;
-            uint64_t u = 0, v = 0, h = 0;
-            for (int l = 0; l < J.scale; ++l) {
-                if ((l & 1) == 0) h = draw(J.key, base + (uint64_t)(l >> 1));
-                const uint32_t r = (l & 1) ? (uint32_t)(h >> 32) : (uint32_t)h;
-                const uint64_t bu = (r >= J.t2) ? 1ull : 0ull;
-                const uint64_t bv = (r >= J.t1 && r < J.t2) || (r >= J.t3) ? 1ull : 0ull;
-                u = (u << 1) | bu;
-                v = (v << 1) | bv;
+//
+// Bound by the draws' arithmetic.  A request's n is rarely a power of two, so
+// an attempt succeeds about six times in ten, and 32 lanes that wait for the
+// last of them make four to five attempts a pair.  So a warp owns a stretch of
+// pairs and a lane whose pair is done takes the stretch's next one.
+__global__ void __launch_bounds__(256) k_rmat_multi(const RmatJob* __restrict__ jobs,
+                                                    const int64_t* __restrict__ ppre, int nreq, int64_t total,
+                                                    int64_t stretch, int32_t* __restrict__ src,
+                                                    int32_t* __restrict__ dst) {
+    const int lane = threadIdx.x & 31;
+    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    int64_t next = warp * stretch;
+    const int64_t end = min64(next + stretch, total);
+    int64_t x = 0, first = 0, last = 0;   // the lane's pair; its request's pairs [first, last)
+    int64_t vbase = 0;
+    RmatShape J{};
+    bool busy = false;
+    int attempt = 0;
+    while (true) {
+        const unsigned idle = __ballot_sync(0xffffffffu, !busy);
+        if (!busy) {
+            x = next + __popc(idle & ((1u << lane) - 1u));
+            busy = x < end;
+            attempt = 0;
+            if (busy && (x < first || x >= last)) {
+                int lo = 0, hi = nreq - 1;
+                while (lo < hi) {
+                    const int mid = (lo + hi + 1) >> 1;
+                    if (ppre[mid] <= x) lo = mid; else hi = mid - 1;
+                }
+                const RmatJob& K = jobs[lo];
+                J = RmatShape{K.key, (uint32_t)K.A, (uint32_t)K.B, (uint32_t)K.C, (uint32_t)K.n, K.t1, K.t2, K.t3,
+                              K.scale};
+                vbase = K.vbase;
+                first = ppre[lo];
+                last = ppre[lo + 1];
             }
-            u = ((((u * J.A) & mask) ^ J.B) * J.C) & mask;
-            v = ((((v * J.A) & mask) ^ J.B) * J.C) & mask;
-            if (u < (uint64_t)J.n && v < (uint64_t)J.n) {
-                su = (int64_t)u;
-                sv = (int64_t)v;
-                break;
+        }
+        next += __popc(idle);
+        if (!__any_sync(0xffffffffu, busy)) break;
+        if (busy) {
+            uint32_t u, v;
+            const bool ok = rmat_attempt(J, (uint64_t)(x - first), attempt, u, v);
+            if (ok || ++attempt == kAttempts) {
+                src[x] = (int32_t)(vbase + (ok ? u : 0u));
+                dst[x] = (int32_t)(vbase + (ok ? v : 0u));
+                busy = false;
             }
         }
-        src[x] = (int32_t)(J.vbase + su);
-        dst[x] = (int32_t)(J.vbase + sv);
     }
 }
 
@@ -126,8 +147,11 @@ void generate_rmat_multi(const RmatJob* jobs_dev, const int64_t* ppre_dev, int n
     if (total <= 0) return;
     {
         Prof prof_("k_rmat_multi", st);
-        k_rmat_multi<<<grid_for(total, 256, (int64_t)num_sms() * 16), 256, 0, st>>>(
-            jobs_dev, ppre_dev, nreq, total, src, dst);
+        // as many warps as the device runs at once, a whole number of rounds each
+        const int64_t warps = std::min<int64_t>((total + 31) / 32, (int64_t)num_sms() * 64);
+        const int64_t stretch = (total + warps - 1) / warps;
+        k_rmat_multi<<<grid_for(32 * ((total + stretch - 1) / stretch), 256), 256, 0, st>>>(
+            jobs_dev, ppre_dev, nreq, total, stretch, src, dst);
     }
     TC_LAUNCH_CHECK();
 }
@@ -162,8 +186,8 @@ extern "C" tc_status tc_generate_rmat(uint64_t seed, int32_t scale, int64_t n, i
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     {
         Prof prof_("k_rmat", st);
-        k_rmat<<<grid_for(count, 256, (int64_t)num_sms() * 16), 256, 0, st>>>(
-        key, scale, (uint64_t)n, e0, count, t1, t2, t3, A, B, C, src_dev, dst_dev);
+        const RmatShape J{key, (uint32_t)A, (uint32_t)B, (uint32_t)C, (uint32_t)n, t1, t2, t3, scale};
+        k_rmat<<<grid_for(count, 256, (int64_t)num_sms() * 16), 256, 0, st>>>(J, e0, count, src_dev, dst_dev);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
