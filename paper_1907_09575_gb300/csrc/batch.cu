@@ -60,18 +60,19 @@ void set_tuning(tc_batch* b, const tc_tuning& t) {
         b->units = UnitLists{};
     }
     b->alloc.stream = b->cap;
-    b->units = build_unit_lists(b->views, b->vpre, b->num, b->V, tt, b->alloc, b->cap);
+    // few tasks a wide unit only while all of the batch's are few
+    b->units = build_unit_lists(b->views, b->vpre, b->num, b->V, unit_rule(tt, false, zone_capacity(m) > 0), b->alloc,
+                                b->cap);
     TC_CUDA(cudaStreamSynchronize(b->cap));
+    for (const tc_graph* g : b->graphs) b->units.zones |= g->zcap > 0;
     b->tuning = tt;
     const CountLaunch c = prepare_count(b->units, tt, false);
-    prepare_mid();
     TC_CUDA(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
     cudaError_t e1 = cudaMemsetAsync(b->ctr, 0, sizeof(unsigned long long) * CTR_COUNT, b->cap);
     cudaError_t e2 = cudaMemsetAsync(b->totals, 0, sizeof(uint64_t) * (size_t)b->num, b->cap);
     bool launched = true;
     try {
         launch_count_raw(c, b->views, b->units, tt, b->ctr, b->cap);
-        launch_mid(b->views, b->units, tt, false, b->ctr, b->cap, nullptr, false);
         launch_zone(b->views, b->units, false, b->ctr, b->cap, nullptr, false);
     } catch (const Error&) {
         launched = false;
@@ -258,28 +259,25 @@ tc_status tc_batch_autotune(tc_batch* b, int32_t reps, tc_tuning* chosen, void* 
         const int warp_tasks[] = {64, 512};
         const int cta_tasks[] = {512, 4096};
         const int threads[] = {128, 256};
-        const int merge_max[] = {0, 16};   // short pivot rows searched instead of tabled
         for (int a : small_max)
             for (int w : warp_tasks)
                 for (int c : cta_tasks)
-                    for (int th : threads)
-                        for (int mm : merge_max) {
-                            tc_tuning cand;
-                            tuning_defaults(&cand);
-                            cand.small_max_outdeg = a;
-                            cand.warp_unit_tasks = w;
-                            cand.cta_unit_tasks = c;
-                            cand.cta_threads = th;
-                            cand.merge_max_outdeg = mm;
-                            tc_tuning res;
-                            tuning_resolve(&cand, &res);
-                            set_tuning(b, res);
-                            const float ms = time_batch(b, std::max(reps, 1), st);
-                            if (ms < best_ms) {
-                                best_ms = ms;
-                                best = b->tuning;
-                            }
+                    for (int th : threads) {
+                        tc_tuning cand;
+                        tuning_defaults(&cand);
+                        cand.small_max_outdeg = a;
+                        cand.warp_unit_tasks = w;
+                        cand.cta_unit_tasks = c;
+                        cand.cta_threads = th;
+                        tc_tuning res;
+                        tuning_resolve(&cand, &res);
+                        set_tuning(b, res);
+                        const float ms = time_batch(b, std::max(reps, 1), st);
+                        if (ms < best_ms) {
+                            best_ms = ms;
+                            best = b->tuning;
                         }
+                    }
         std::lock_guard<std::mutex> lk(g_tune_mu);
         g_tune_cache[sig] = best;
     }

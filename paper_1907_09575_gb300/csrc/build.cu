@@ -33,7 +33,6 @@
 
 #include "common.cuh"
 #include "tc_internal.cuh"
-#include "zone.cuh"
 
 namespace tc {
 namespace {
@@ -100,8 +99,8 @@ struct BuildArgs {
     int64_t zcap;
     GraphView view, view_comp;
     GraphView *view_at, *view_comp_at;
-    Unit *small, *large, *zone;
-    int small_max, warp_tasks, cta_tasks, slice_max;
+    Unit *large, *wide;      // the small units follow the wide ones
+    UnitRule rule;
 };
 
 enum : int { kPhaseInsert = 0, kPhaseGraph = 1, kPhaseUnits = 2, kPhaseEnd = 3 };
@@ -694,24 +693,15 @@ __device__ void phase_sort(const BuildArgs& a, uint32_t* smem) {
 }
 
 // --- tasks and units ----------------------------------------------------------
-__device__ __forceinline__ void unit_counts(const BuildArgs& a, long long dp, long long nt, long long& small,
-                                            long long& large, long long& zone) {
-    small = large = 0;
-    zone = a.zcap > 0 && dp > kZoneMinPivot ? (nt + kZoneTasks - 1) / kZoneTasks : 0;
-    if (dp > 0 && nt > 0) {
-        if (dp <= a.small_max) small = (nt + a.warp_tasks - 1) / a.warp_tasks;
-        else if (zone == 0 || dp > kMidMaxOutdeg) large = ((dp + a.slice_max - 1) / a.slice_max) * ((nt + a.cta_tasks - 1) / a.cta_tasks);
-    }
-}
-
 __device__ void tasks_sum(const BuildArgs& a) {
     if ((int)blockIdx.x >= a.nchunks) return;
     const int64_t c0 = (int64_t)blockIdx.x * a.chunk, c1 = min64(c0 + a.chunk, a.n);
     long long t = 0, us = 0, ul = 0, uz = 0, total;
     for (int64_t r = c0 + threadIdx.x; r < c1; r += kBT) {
-        long long x, y, z, nt = 0;
+        long long nt = 0;
+        int64_t x, y, z;
         for (int c = 0; c < a.tcopies; ++c) nt += a.tcur[c * a.n + r];
-        unit_counts(a, a.dplus[r], nt, x, y, z);
+        unit_split(a.rule, a.zcap > 0, a.dplus[r], nt, x, y, z);
         t += nt;
         us += x;
         ul += y;
@@ -827,7 +817,7 @@ __device__ void tasks_write(const BuildArgs& a) {
     if ((threadIdx.x & 31) == 0 && cut) atomicAdd(&a.tally->covered, cut);
 }
 
-__device__ __forceinline__ void put_unit(const BuildArgs& a, int64_t j, bool small, long long at, int64_t q,
+__device__ __forceinline__ void put_unit(const BuildArgs& a, Unit* small_at, int64_t j, bool small, long long at, int64_t q,
                                          int64_t slices, int64_t t0, int64_t t1) {
     Unit u;
     u.j = (int32_t)j;
@@ -835,13 +825,13 @@ __device__ __forceinline__ void put_unit(const BuildArgs& a, int64_t j, bool sma
     u.pad = 0;
     if (small) {
         u.slice = 0;
-        u.t0 = t0 + q * a.warp_tasks;
-        u.t1 = min64(u.t0 + a.warp_tasks, t1);
-        a.small[at + q] = u;
+        u.t0 = t0 + q * a.rule.warp_tasks;
+        u.t1 = min64(u.t0 + a.rule.warp_tasks, t1);
+        small_at[at + q] = u;
     } else {
         u.slice = (int32_t)(q % slices);
-        u.t0 = t0 + q / slices * a.cta_tasks;
-        u.t1 = min64(u.t0 + a.cta_tasks, t1);
+        u.t0 = t0 + q / slices * a.rule.cta_tasks;
+        u.t1 = min64(u.t0 + a.rule.cta_tasks, t1);
         a.large[at + q] = u;
     }
 }
@@ -863,14 +853,15 @@ __device__ void phase_units(const BuildArgs& a) {
     const long long ns = a.tally->nsmall, nl = a.tally->nlarge, nz = a.tally->nzone;
     for (int64_t t0 = c0; t0 < c1; t0 += kBT) {
         const int64_t j = t0 + threadIdx.x;
-        long long us = 0, ul = 0, uz = 0, ts, tl, tz;
+        int64_t us = 0, ul = 0, uz = 0;
+        long long ts, tl, tz;
         int64_t b0 = 0, b1 = 0, slices = 1;
         if (j < c1) {
             const int64_t dp = row_begin(a, j + 1) - row_begin(a, j);
             b0 = a.loff[j];
             b1 = a.loff[j + 1];
-            unit_counts(a, dp, b1 - b0, us, ul, uz);
-            slices = (dp + a.slice_max - 1) / a.slice_max;
+            unit_split(a.rule, a.zcap > 0, dp, b1 - b0, us, ul, uz);
+            slices = (dp + a.rule.slice - 1) / a.rule.slice;
         }
         const long long xs = cs + block_scan(us, &ts), xl = cl + block_scan(ul, &tl);
         const long long az = nz - uz - (cz + block_scan(uz, &tz));
@@ -881,7 +872,7 @@ __device__ void phase_units(const BuildArgs& a) {
         const long long count = us + ul;
         const long long at = small ? ns - xs - us : nl - xl - ul;
         if (count > 0 && count <= kBItems)
-            for (int64_t q = 0; q < count; ++q) put_unit(a, j, small, at, q, slices, b0, b1);
+            for (int64_t q = 0; q < count; ++q) put_unit(a, a.wide + nz, j, small, at, q, slices, b0, b1);
         unsigned many = __ballot_sync(0xffffffffu, count > kBItems);
         while (many) {
             const int o = __ffs(many) - 1;
@@ -890,7 +881,7 @@ __device__ void phase_units(const BuildArgs& a) {
             const int64_t x0 = __shfl_sync(0xffffffffu, b0, o), x1 = __shfl_sync(0xffffffffu, b1, o);
             const int64_t s = __shfl_sync(0xffffffffu, slices, o), jj = __shfl_sync(0xffffffffu, j, o);
             const bool sm = __shfl_sync(0xffffffffu, (int)small, o);
-            for (int64_t q = lane; q < c; q += 32) put_unit(a, jj, sm, p, q, s, x0, x1);
+            for (int64_t q = lane; q < c; q += 32) put_unit(a, a.wide + nz, jj, sm, p, q, s, x0, x1);
         }
         unsigned zoned = __ballot_sync(0xffffffffu, uz > 0);
         while (zoned) {
@@ -900,7 +891,8 @@ __device__ void phase_units(const BuildArgs& a) {
             const int64_t x0 = __shfl_sync(0xffffffffu, b0, o), x1 = __shfl_sync(0xffffffffu, b1, o);
             const int64_t jj = __shfl_sync(0xffffffffu, j, o);
             for (int64_t q = lane; q < c; q += 32)
-                a.zone[p + q] = Unit{(int32_t)jj, 0, 0, 0, x0 + q * kZoneTasks, min64(x0 + (q + 1) * kZoneTasks, x1)};
+                a.wide[p + q] =
+                    Unit{(int32_t)jj, 0, 0, 0, x0 + q * a.rule.wide_tasks, min64(x0 + (q + 1) * a.rule.wide_tasks, x1)};
         }
     }
 }
@@ -1064,35 +1056,33 @@ void build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64_t P,
     graph_views(g, &a.view, &a.view_comp);
     a.view_at = g->view;
     a.view_comp_at = g->view_comp;
-    a.small_max = tt.small_max_outdeg;
-    a.warp_tasks = tt.warp_unit_tasks;
-    a.cta_tasks = tt.cta_unit_tasks;
-    a.slice_max = tt.slice_max;
+    a.rule = unit_rule(tt, false, g->zcap > 0);
     UnitLists L;
-    auto take_units = [&](int64_t ns, int64_t nl, int64_t nz) {
-        L.bytes = sizeof(Unit) * (size_t)std::max<int64_t>(ns + nl + nz, 1);
+    auto take_units = [&](int64_t nl, int64_t rest) {
+        L.bytes = sizeof(Unit) * (size_t)std::max<int64_t>(nl + rest, 1);
         L.mem = al.get(L.bytes);
         a.large = L.large = static_cast<Unit*>(L.mem);
-        a.small = L.small = L.large + nl;
-        a.zone = L.zone = L.small + ns;
+        a.wide = L.zone = L.large + nl;
         // the graph owns them from here on, whatever fails next
         adopt_units(g, L, tt);
     };
     if (one) {
-        // every pivot with a task has a unit of its own and at most one more
-        // for each full unit of tasks; a large pivot has over kSmallMaxOutdeg
-        // of the edges, and one slice (d^2 <= 2m)
+        // A large pivot has over kSmallMaxOutdeg of the edges and one slice
+        // (d^2 <= 2m).  Of the others each has a unit, small or wide, and at
+        // most one more for each full unit of tasks; the large ones with
+        // zones are wide as well.
         static_assert(2 * kBuildOnePairs <= (int64_t)kMaxSlice * kMaxSlice, "one slice a pivot");
-        take_units(std::min(n, P) + P / tt.warp_unit_tasks + 1, P / kSmallMaxOutdeg + P / tt.cta_unit_tasks + 1,
-                   P / kZoneMinPivot + P / kZoneTasks + 1);
+        const int64_t nl = P / kSmallMaxOutdeg + P / a.rule.cta_tasks + 1;
+        take_units(nl, std::min(n, P) + P / a.rule.warp_tasks + 2 * (P / a.rule.wide_tasks) + P / kMidMaxOutdeg + 1);
         launch(kPhaseInsert, kPhaseEnd);
         read_tally();
     } else {
         launch(kPhaseGraph, kPhaseUnits);
         read_tally();
-        take_units((int64_t)h.nsmall, (int64_t)h.nlarge, (int64_t)h.nzone);
+        take_units((int64_t)h.nlarge, (int64_t)(h.nsmall + h.nzone));
         launch(kPhaseUnits, kPhaseEnd);
     }
+    g->small_units = g->zone_units + h.nzone;
     g->n_small = h.nsmall;
     g->n_large = h.nlarge;
     g->n_zone = h.nzone;

@@ -27,10 +27,10 @@
 // Per-vertex counts (t[v] = triangles through v): a task's hits credit i once,
 // per-entry hit counters credit k once per unit, j is credited once per unit.
 #include <algorithm>
+#include <memory>
 
 #include "common.cuh"
 #include "tc_internal.cuh"
-#include "zone.cuh"
 
 namespace tc {
 namespace {
@@ -315,28 +315,6 @@ struct MidTab {
     __device__ __forceinline__ unsigned credited(const unsigned* cnt, int r) const { return cnt[r]; }
 };
 
-// Search (the list-based joint traversal of Section 3.1, lane-parallel): the
-// sorted pivot row U_j (at most 64 entries) sits in shared memory and each
-// lane places its probe in it by a branchless binary search.  No table is
-// built; the position found is the entry's index, so per-vertex credit
-// needs no rank.
-struct SearchTab {
-    const int* piv;
-    int dp, lo, hi;
-    template <bool PV>
-    __device__ __forceinline__ int find(int k) const {
-        if ((unsigned)(k - lo) > (unsigned)(hi - lo)) return -1;
-        int pos = 0;
-#pragma unroll
-        for (int step = 32; step > 0; step >>= 1)
-            if (pos + step < dp && piv[pos + step] <= k) pos += step;
-        return piv[pos] == k ? pos : -1;
-    }
-    __device__ __forceinline__ unsigned bit(int k) const { return find<false>(k) >= 0; }
-    __device__ __forceinline__ void credit(unsigned* cnt, int r) const { atomicAdd(&cnt[r], 1u); }
-    __device__ __forceinline__ unsigned credited(const unsigned* cnt, int r) const { return cnt[r]; }
-};
-
 __device__ __forceinline__ void hash_insert(int* tab, unsigned bmask, int k) {
     unsigned b = (unsigned)k & bmask;
     while (true) {
@@ -599,9 +577,9 @@ struct GraphAcc {
 // Warp unit: a pivot with |U_j| <= 64 processed by one warp with a private
 // table (a bitmap of <= 4095 labels, or 128 hash slots).
 // ---------------------------------------------------------------------------
-template <bool PV, bool MERGE, bool WIN>
+template <bool PV, bool WIN>
 __device__ __forceinline__ void warp_unit(const GraphView& G, const Unit& U, unsigned* region,
-                                          unsigned* cnt, int64_t* s_base, bool hash_only, int merge_max,
+                                          unsigned* cnt, int64_t* s_base, bool hash_only,
                                           unsigned* tlow, uint64_t& hits, uint64_t& probes, uint64_t& staged) {
     const int lane = threadIdx.x & 31;
     const int64_t rb = off_at(G, U.j), re = off_at(G, U.j + 1);
@@ -613,27 +591,7 @@ __device__ __forceinline__ void warp_unit(const GraphView& G, const Unit& U, uns
     uint64_t uh = 0;
     if (PV)
         for (int s = lane; s < kSmallTable / 2; s += 32) cnt[s] = 0;
-    if (MERGE && dp <= merge_max) {
-        int* piv = reinterpret_cast<int*>(region);
-        if (lane < dp) piv[lane] = mine;
-        if (lane + 32 < dp) piv[lane + 32] = mine2;
-        __syncwarp();
-        const SearchTab T{piv, dp, lo, hi};
-        for (int64_t tb = U.t0; tb < U.t1; tb += 32)
-            warp_probe_group<PV, WIN>(G.tasks, tb, U.t1, G.adj, T, cnt, G.tnew, tlow, s_base, U.t0, nullptr,
-                                      nullptr, uh, probes, TaskWindow{G.i0, G.i1, G.tail_shift});
-        __syncwarp();
-        if (PV) {
-            if (lane < dp) {
-                const unsigned h = T.credited(cnt, lane);
-                if (h) atomicAdd(&G.tnew[mine], (unsigned long long)h);
-            }
-            if (lane + 32 < dp) {
-                const unsigned h = T.credited(cnt, lane + 32);
-                if (h) atomicAdd(&G.tnew[mine2], (unsigned long long)h);
-            }
-        }
-    } else if (bitmap) {
+    if (bitmap) {
         const int words = ((hi - lo + 1) >> 5) + 1;
         for (int s = lane; s < words; s += 32) region[s] = 0;
         __syncwarp();
@@ -945,11 +903,10 @@ __device__ __forceinline__ void cta_unit(const GraphView& G, const Unit& U, int 
 // kTagMaxEntries of them; totals only: the second table alone) | long-task
 // queue (unit_tasks x 16 bit).
 // ---------------------------------------------------------------------------
-template <bool PV, bool MERGE, bool WIN, bool BUCKETS>
+template <bool PV, bool WIN, bool BUCKETS>
 __global__ void __launch_bounds__(256, TC_LARGE_MINB)
     k_count(const GraphView* __restrict__ views, const Unit* __restrict__ large, int64_t nlarge,
-            const Unit* __restrict__ small, int64_t nsmall, int slice_max, int table_mode,
-            int merge_max, int grab, unsigned* tlow,
+            const Unit* __restrict__ small, int64_t nsmall, int slice_max, int grab, unsigned* tlow,
             unsigned long long* __restrict__ ctr) {
     extern __shared__ __align__(16) unsigned smem[];
     __shared__ long long s_unit;
@@ -993,11 +950,12 @@ __global__ void __launch_bounds__(256, TC_LARGE_MINB)
     if (lane == 0 && probes) atomicAdd(&ctr[CTR_PROBES + 1], (unsigned long long)probes);
     probes = 0;
 
-    // warp units, each warp on its own slice of the region
+    // warp units, each warp on its own slice of the region (k_light's in the
+    // ordinary instance)
     unsigned* wregion = region + w * kSmallRegionWords;
     unsigned* wcnt = cnt + w * (kSmallTable / 2);
     uint64_t staged = 0;
-    while (true) {
+    while (WIN || BUCKETS) {
         long long u0 = 0;
         if (lane == 0) u0 = (long long)atomicAdd(&ctr[CTR_SMALL_HEAD], (unsigned long long)grab);
         u0 = __shfl_sync(0xffffffffu, u0, 0);
@@ -1007,7 +965,7 @@ __global__ void __launch_bounds__(256, TC_LARGE_MINB)
             const Unit U = small[u];
             const GraphView G = views[U.g];
             acc.to(unit_target(G, U));
-            warp_unit<PV, MERGE, WIN>(G, U, wregion, wcnt, s_base, BUCKETS, merge_max, tlow, acc.hits,
+            warp_unit<PV, WIN>(G, U, wregion, wcnt, s_base, BUCKETS, tlow, acc.hits,
                                  probes, staged);
             if (lane == 0) {
                 atomicAdd(&s_work[0], 1ull);
@@ -1044,7 +1002,25 @@ __global__ void __launch_bounds__(256, TC_LARGE_MINB)
 // ---------------------------------------------------------------------------
 constexpr int kMidThreads = 256;
 constexpr int kMidBitWords = (kMidSlots * 2 / 3) & ~31;
+constexpr int kLightMinBlocks = 4;
 constexpr size_t mid_warp_words(bool pv) { return 64 + kMidSlots + kMidSlots2 + (pv ? kMidEntries : 0); }
+
+constexpr size_t light_smem(bool pv) { return sizeof(unsigned) * mid_warp_words(pv) * (kMidThreads / 32); }
+
+constexpr int kFlatUnits = 4;
+static_assert(kFlatUnits * kSmallMaxOutdeg <= kMidEntries, "the units' counters fit the pivot counters of a warp");
+constexpr int kFlatWindow = 2048;   // concatenated entries whose tasks' starts are marked at once
+struct __align__(16) FlatWarp {   // one warp's shared memory while it counts warp units
+    int64_t t0[kFlatUnits];   // per unit: first task less the tasks of earlier units
+    const int32_t* adj[kFlatUnits];
+    unsigned heads[kFlatWindow / 32];   // bit q: a task's entries start at q
+    int row[kFlatUnits * kSmallMaxOutdeg];   // the pivots' rows, filled up with the largest int
+    int end[kFlatUnits];      // tasks up to and including the unit's
+    unsigned rb[kFlatUnits];
+    int j[kFlatUnits], g[kFlatUnits];
+    unsigned base[32];        // per task with a tail: its entries' place less their position
+    int unit[32];             // its unit
+};
 
 template <bool PV, class Tab>
 __device__ __forceinline__ void mid_probe(const GraphView& G, const Unit& U, const Tab& T, unsigned* cnt,
@@ -1067,17 +1043,204 @@ __device__ __forceinline__ void mid_probe(const GraphView& G, const Unit& U, con
     }
 }
 
+// Pivots of at most kSmallMaxOutdeg entries (warp units), without tables: the
+// tasks of up to kFlatUnits units are dealt to the lanes 32 at a time whatever
+// their pivots, their tails concatenated, and each entry is looked up by a
+// branchless binary search of its own pivot's row in shared memory (the
+// list-based traversal of Section 3.1, a lane a probe).  Such a unit holds
+// some hundred probes: as a table of its own, built, probed and flushed, it
+// took 600-1,000 instructions whatever its size (G(n,p) of 1.6e6 edges:
+// 141,601 units, 146 us).  An entry's task is the number of task starts up to
+// it, counted in a bit mask of the starts.  Few units at a time: a hub's are
+// hundreds of times longer than others.  Per-vertex: hits on the pivots'
+// entries count in shared memory (adding each to its vertex's accumulator
+// made the hubs' a bottleneck: RMAT scale 20 0.7 -> 2.3 ms).
 template <bool PV>
-__global__ void __launch_bounds__(kMidThreads, 4)
-    k_mid(const GraphView* __restrict__ views, const Unit* __restrict__ units, int64_t nunits, unsigned* tlow,
-          unsigned long long* __restrict__ ctr) {
+__device__ __forceinline__ void flat_units(const GraphView* __restrict__ views, const Unit* __restrict__ small,
+                                           long long u0, int n, FlatWarp& S, unsigned* cnt, unsigned* tlow,
+                                           GraphAcc& acc, unsigned long long* work) {
+    const int lane = threadIdx.x & 31;
+    const unsigned le = (2u << lane) - 1u;
+    int nt = 0, dp = 0;
+    Unit U{};
+    __syncwarp();   // the last batch's reads of S are done
+    if (lane < n) {
+        U = small[u0 + lane];
+        const GraphView& V = views[U.g];
+        const int64_t rb = off_at(V, U.j);
+        dp = (int)(off_at(V, U.j + 1) - rb);
+        nt = (int)(U.t1 - U.t0);
+        S.adj[lane] = V.adj;
+        S.rb[lane] = (unsigned)rb;
+        S.j[lane] = U.j;
+        S.g[lane] = U.g;
+    }
+    const int uend = warp_incl_scan_i32(nt);
+    const int N = __shfl_sync(0xffffffffu, uend, 31);
+    if (lane < kFlatUnits) {
+        S.end[lane] = lane < n ? uend : 0x7fffffff;
+        S.t0[lane] = U.t0 - (uend - nt);
+    }
+    const int g0 = __shfl_sync(0xffffffffu, U.g, 0);
+    const bool one_graph = __all_sync(0xffffffffu, lane >= n || U.g == g0);
+    const bool wide_rows = __any_sync(0xffffffffu, dp > 16);
+    const int32_t* __restrict__ adj0 = views[g0].adj;
+    // hits may go to one counter as they come, without a task's share of them
+    const bool bulk = !PV && one_graph && !views[g0].comp;
+    if (bulk) acc.to(views[g0].total);
+    __syncwarp();
+#pragma unroll
+    for (int o = 0; o < kFlatUnits; ++o) {
+        if (o >= n) break;
+        const int d = __shfl_sync(0xffffffffu, dp, o);
+        const int32_t* a = S.adj[o] + S.rb[o];
+        int* r = S.row + o * kSmallMaxOutdeg;
+        r[lane] = lane < d ? a[lane] : 0x7fffffff;
+        r[lane + 32] = lane + 32 < d ? a[lane + 32] : 0x7fffffff;
+        if (PV) {
+            cnt[o * kSmallMaxOutdeg + lane] = 0;
+            cnt[o * kSmallMaxOutdeg + lane + 32] = 0;
+        }
+    }
+    __syncwarp();
+    unsigned nprobes = 0;
+    for (int x0 = 0; x0 < N; x0 += 32) {
+        const int x = x0 + lane;
+        // this lane's task and its unit: the first that ends after x
+        int o = 0;
+#pragma unroll
+        for (int step = kFlatUnits / 2; step > 0; step >>= 1)
+            if (S.end[o + step - 1] <= x) o += step;
+        o = min(o, n - 1);
+        int len = 0, i = 0;
+        unsigned start = 0;
+        if (x < N) {
+            const Task t = views[S.g[o]].tasks[S.t0[o] + x];
+            start = t.start;
+            len = t.len;
+            i = t.i;
+        }
+        const int incl = warp_incl_scan_i32(len), excl = incl - len;
+        const int total = __shfl_sync(0xffffffffu, incl, 31);
+        const unsigned on = __ballot_sync(0xffffffffu, len > 0);
+        if (len > 0) {
+            const int at = __popc(on & (le >> 1));
+            S.base[at] = start - (unsigned)excl;
+            S.unit[at] = o;
+        }
+        nprobes += (unsigned)total;
+        unsigned c = 0;
+        for (int w0 = 0; w0 < total; w0 += kFlatWindow) {
+            S.heads[lane] = 0;
+            S.heads[lane + 32] = 0;
+            __syncwarp();
+            if (len > 0 && excl >= w0 && excl < w0 + kFlatWindow)
+                atomicOr(&S.heads[(excl - w0) >> 5], 1u << (excl & 31));
+            int seen = __popc(__ballot_sync(0xffffffffu, len > 0 && excl < w0)) - 1;
+            __syncwarp();
+            const int w1 = min(total, w0 + kFlatWindow);
+            for (int q0 = w0; q0 < w1; q0 += 32 * kUnroll) {
+                static_assert(kUnroll == 4, "four words of starts a round");
+                const uint4 H = *reinterpret_cast<const uint4*>(&S.heads[(q0 - w0) >> 5]);
+                const unsigned M[4] = {H.x, H.y, H.z, H.w};
+                int k[kUnroll], p[kUnroll];
+#pragma unroll
+                for (int u = 0; u < kUnroll; ++u) {
+                    const int q = q0 + 32 * u + lane;
+                    const int w = seen + __popc(M[u] & le);
+                    seen += __popc(M[u]);
+                    k[u] = -1;
+                    p[u] = 0;
+                    if (q < w1) {
+                        const int un = S.unit[w];
+                        const int32_t* __restrict__ a = one_graph ? adj0 : S.adj[un];
+                        k[u] = __ldg(a + (S.base[w] + (unsigned)q));
+                        p[u] = un * kSmallMaxOutdeg;
+                    }
+                }
+                // the last entry <= k
+                if (wide_rows) {
+#pragma unroll
+                    for (int u = 0; u < kUnroll; ++u)
+                        if (S.row[p[u] + 32] <= k[u]) p[u] += 32;
+#pragma unroll
+                    for (int u = 0; u < kUnroll; ++u)
+                        if (S.row[p[u] + 16] <= k[u]) p[u] += 16;
+                }
+#pragma unroll
+                for (int s = 8; s > 0; s >>= 1) {
+#pragma unroll
+                    for (int u = 0; u < kUnroll; ++u)
+                        if (S.row[p[u] + s] <= k[u]) p[u] += s;
+                }
+#pragma unroll
+                for (int u = 0; u < kUnroll; ++u) {
+                    const bool hit = S.row[p[u]] == k[u];
+                    if (PV && hit) atomicAdd(&cnt[p[u]], 1u);
+                    if (bulk) {
+                        acc.hits += hit ? 1 : 0;
+                    } else {
+                        const unsigned hm = __ballot_sync(0xffffffffu, hit);
+                        if (hm) {   // each task takes its hits of these 32
+                            const int qb = q0 + 32 * u;
+                            const int b0 = max(excl - qb, 0), b1 = min(incl - qb, 32);
+                            if (b0 < b1) c += __popc(hm & bit_range(b0, b1));
+                        }
+                    }
+                }
+            }
+            __syncwarp();
+        }
+        if (!bulk) {
+            // credits: per task, and per unit for its pivot and total
+            const GraphView& V = views[S.g[o]];
+            if (PV && c) credit_task(V.tnew, tlow, i, c);
+            const int csum = warp_incl_scan_i32((int)c);
+            const int o_next = __shfl_down_sync(0xffffffffu, o, 1);
+            const bool seg_end = x < N && (lane == 31 || x + 1 == N || o_next != o);
+            const unsigned ends = __ballot_sync(0xffffffffu, seg_end);
+            const unsigned below = ends & (le >> 1);
+            const int prev = __shfl_sync(0xffffffffu, csum, below ? 31 - __clz(below) : 0);
+            const unsigned h = (unsigned)(csum - (below ? prev : 0));
+            if (seg_end && h) {
+                if (PV) atomicAdd(&V.tnew[S.j[o]], (unsigned long long)h);
+                atomicAdd(V.comp ? V.comp_totals + V.comp[S.j[o]] : V.total, (unsigned long long)h);
+            }
+        }
+        __syncwarp();   // base and unit are rewritten by the next 32 tasks
+    }
+    if (PV) {
+        for (int q = lane; q < n * kSmallMaxOutdeg; q += 32) {
+            const unsigned h = cnt[q];
+            if (h) atomicAdd(&views[S.g[q / kSmallMaxOutdeg]].tnew[S.row[q]], (unsigned long long)h);
+        }
+    }
+    const unsigned staged = __reduce_add_sync(0xffffffffu, (unsigned)dp);
+    if (lane == 0) {
+        work[0] += (unsigned)n;
+        work[1] += (unsigned)N;
+        work[2] += nprobes;
+        work[3] += staged;
+    }
+}
+
+static_assert(sizeof(FlatWarp) <= sizeof(unsigned) * (64 + kMidSlots + kMidSlots2) && mid_warp_words(true) % 4 == 0 &&
+                  mid_warp_words(false) % 4 == 0, "one region, 16-byte aligned, for both parts");
+
+template <bool PV>
+__global__ void __launch_bounds__(kMidThreads, kLightMinBlocks)
+    k_light(const GraphView* __restrict__ views, const Unit* __restrict__ units, int64_t nunits,
+            const Unit* __restrict__ small, int64_t nsmall, int grab, unsigned* tlow,
+            unsigned long long* __restrict__ ctr) {
     extern __shared__ __align__(16) unsigned smem[];
+    __shared__ unsigned long long s_work[kMidThreads / 32][4];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     unsigned* mine = smem + (size_t)w * mid_warp_words(PV);
     int64_t* s_base = reinterpret_cast<int64_t*>(mine);
     unsigned* tab = mine + 64;
     unsigned* t2 = tab + kMidSlots;
     unsigned* cnt = t2 + kMidSlots2;
+    if (lane < 4) s_work[w][lane] = 0;
     GraphAcc acc;
     uint64_t probes = 0, staged = 0;
     unsigned long long nu = 0, nt = 0;
@@ -1150,12 +1313,26 @@ __global__ void __launch_bounds__(kMidThreads, 4)
         nt += (unsigned long long)(U.t1 - U.t0);
         __syncwarp();   // the table is rebuilt by the next unit
     }
-    acc.flush();
     if (lane == 0 && nu) {
         atomicAdd(&ctr[CTR_UNITS + 1], nu);
         atomicAdd(&ctr[CTR_TASKS + 1], nt);
         atomicAdd(&ctr[CTR_PROBES + 1], (unsigned long long)probes);
         atomicAdd(&ctr[CTR_STAGED + 1], (unsigned long long)staged);
+    }
+    // the warp units
+    FlatWarp& S = *reinterpret_cast<FlatWarp*>(mine);
+    while (true) {
+        long long u0 = 0;
+        if (lane == 0) u0 = (long long)atomicAdd(&ctr[CTR_SMALL_HEAD], (unsigned long long)grab);
+        u0 = __shfl_sync(0xffffffffu, u0, 0);
+        if (u0 >= nsmall) break;
+        flat_units<PV>(views, small, u0, (int)min64(grab, nsmall - u0), S, cnt, tlow, acc, s_work[w]);
+    }
+    acc.flush();
+    __syncwarp();
+    if (lane < 4 && s_work[w][0]) {
+        const int slot = lane == 0 ? CTR_UNITS : lane == 1 ? CTR_TASKS : lane == 2 ? CTR_PROBES : CTR_STAGED;
+        atomicAdd(&ctr[slot], s_work[w][lane]);
     }
 }
 
@@ -1191,33 +1368,24 @@ __device__ __forceinline__ int find_graph(const int64_t* __restrict__ vpre, int 
 }
 
 __global__ void k_unit_counts(const GraphView* __restrict__ views, const int64_t* __restrict__ vpre,
-                              int num, int64_t V, int small_max, int mid_max, int tw, int tcta, int slice,
-                              int32_t* __restrict__ cs, int32_t* __restrict__ cl, int32_t* __restrict__ cz) {
+                              int num, int64_t V, UnitRule rule, int32_t* __restrict__ cs,
+                              int32_t* __restrict__ cl, int32_t* __restrict__ cz) {
     for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < V;
          x += (int64_t)gridDim.x * blockDim.x) {
         const int64_t v = V - 1 - x;
         const int g = find_graph(vpre, num, v);
         const GraphView& G = views[g];
         const int64_t j = v - vpre[g];
-        const int64_t dp = off_at(G, j + 1) - off_at(G, j);
-        const int64_t nt = G.loff[j + 1] - G.loff[j];
-        int32_t a = 0, b = 0;
-        cz[x] = G.zrow && dp > kZoneMinPivot ? (int32_t)((nt + kZoneTasks - 1) / kZoneTasks) : 0;
-        if (dp > 0 && nt > 0) {
-            if (dp <= small_max) {
-                a = (int32_t)((nt + tw - 1) / tw);
-            } else if (!(G.zrow && dp > kZoneMinPivot && dp <= mid_max)) {
-                const int64_t slices = (dp + slice - 1) / slice;
-                b = (int32_t)(slices * ((nt + tcta - 1) / tcta));
-            }
-        }
-        cs[x] = a;
-        cl[x] = b;
+        int64_t a, b, c;
+        unit_split(rule, G.zrow != nullptr, off_at(G, j + 1) - off_at(G, j), G.loff[j + 1] - G.loff[j], a, b, c);
+        cs[x] = (int32_t)a;
+        cl[x] = (int32_t)b;
+        cz[x] = (int32_t)c;
     }
 }
 
 __global__ void k_unit_fill(const GraphView* __restrict__ views, const int64_t* __restrict__ vpre,
-                            int num, int64_t V, int small_max, int mid_max, int tw, int tcta, int slice,
+                            int num, int64_t V, UnitRule rule,
                             const int64_t* __restrict__ ps, const int64_t* __restrict__ pl,
                             const int64_t* __restrict__ pz, Unit* __restrict__ us, Unit* __restrict__ ul,
                             Unit* __restrict__ uz) {
@@ -1229,27 +1397,39 @@ __global__ void k_unit_fill(const GraphView* __restrict__ views, const int64_t* 
         const int64_t j = v - vpre[g];
         const int64_t dp = off_at(G, j + 1) - off_at(G, j);
         const int64_t a = G.loff[j], b = G.loff[j + 1];
-        if (dp <= 0 || b <= a) continue;
-        if (G.zrow && dp > kZoneMinPivot) {
+        int64_t ns, nl, nw;
+        unit_split(rule, G.zrow != nullptr, dp, b - a, ns, nl, nw);
+        if (nw > 0) {
             int64_t p = pz[x];
-            for (int64_t t = a; t < b; t += kZoneTasks)
-                uz[p++] = Unit{(int32_t)j, 0, g, 0, t, min64(t + kZoneTasks, b)};
+            for (int64_t t = a; t < b; t += rule.wide_tasks)
+                uz[p++] = Unit{(int32_t)j, 0, g, 0, t, min64(t + rule.wide_tasks, b)};
         }
-        if (dp <= small_max) {
+        if (ns > 0) {
             int64_t p = ps[x];
-            for (int64_t t = a; t < b; t += tw)
-                us[p++] = Unit{(int32_t)j, 0, g, 0, t, min64(t + tw, b)};
-        } else if (!(G.zrow && dp > kZoneMinPivot && dp <= mid_max)) {
-            const int64_t slices = (dp + slice - 1) / slice;
+            for (int64_t t = a; t < b; t += rule.warp_tasks)
+                us[p++] = Unit{(int32_t)j, 0, g, 0, t, min64(t + rule.warp_tasks, b)};
+        } else if (nl > 0) {
+            const int64_t slices = (dp + rule.slice - 1) / rule.slice;
             int64_t p = pl[x];
-            for (int64_t t = a; t < b; t += tcta)
+            for (int64_t t = a; t < b; t += rule.cta_tasks)
                 for (int64_t s = 0; s < slices; ++s)
-                    ul[p++] = Unit{(int32_t)j, (int32_t)s, g, 0, t, min64(t + tcta, b)};
+                    ul[p++] = Unit{(int32_t)j, (int32_t)s, g, 0, t, min64(t + rule.cta_tasks, b)};
         }
     }
 }
 
 }  // namespace
+
+UnitRule unit_rule(const tc_tuning& t, bool win, bool zones) {
+    UnitRule r;
+    r.small_max = t.small_max_outdeg;
+    r.mid_max = win || t.table_mode == 1 ? 0 : kMidMaxOutdeg;
+    r.warp_tasks = t.warp_unit_tasks;
+    r.cta_tasks = t.cta_unit_tasks;
+    r.wide_tasks = wide_unit_tasks(zones);
+    r.slice = t.slice_max;
+    return r;
+}
 
 tc_tuning clamp_tuning(const tc_tuning& t) {
     tc_tuning tt = t;
@@ -1258,13 +1438,13 @@ tc_tuning clamp_tuning(const tc_tuning& t) {
 }
 
 void plan_units(UnitPlan& P, const GraphView* views_dev, const int64_t* vpre_dev, int num, int64_t V,
-                const tc_tuning& t, Alloc& al, cudaStream_t st) {
+                const UnitRule& rule, Alloc& al, cudaStream_t st) {
     const unsigned G = (unsigned)(num_sms() * 8);
     P.V = V;
     P.num = num;
     P.views = views_dev;
     P.vpre = vpre_dev;
-    P.t = t;
+    P.rule = rule;
     P.cs = Buf<int32_t>(al, (size_t)std::max<int64_t>(V, 1));
     P.cl = Buf<int32_t>(al, (size_t)std::max<int64_t>(V, 1));
     P.cz = Buf<int32_t>(al, (size_t)std::max<int64_t>(V, 1));
@@ -1273,10 +1453,8 @@ void plan_units(UnitPlan& P, const GraphView* views_dev, const int64_t* vpre_dev
     P.pz = Buf<int64_t>(al, (size_t)(V + 1));
     if (V > 0) {
         Prof prof_("k_unit_counts", st);
-        k_unit_counts<<<grid_for(V, 256, G), 256, 0, st>>>(views_dev, vpre_dev, num, V,
-                                                           t.small_max_outdeg, mid_max_outdeg(t), t.warp_unit_tasks,
-                                                           t.cta_unit_tasks, t.slice_max, P.cs.get(),
-                                                           P.cl.get(), P.cz.get());
+        k_unit_counts<<<grid_for(V, 256, G), 256, 0, st>>>(views_dev, vpre_dev, num, V, rule, P.cs.get(), P.cl.get(),
+                                                           P.cz.get());
     }
     TC_LAUNCH_CHECK();
     exclusive_scan2_i32_to_i64(P.cs.get(), P.ps.get(), P.ps.get() + V, P.cl.get(), P.pl.get(), P.pl.get() + V, V,
@@ -1298,9 +1476,8 @@ UnitLists fill_units(UnitPlan& P, int64_t ns, int64_t nl, int64_t nz, Alloc& al,
     if (P.V > 0) {
         {
             Prof prof_("k_unit_fill", st);
-            k_unit_fill<<<grid_for(P.V, 256, G), 256, 0, st>>>(
-                P.views, P.vpre, P.num, P.V, P.t.small_max_outdeg, mid_max_outdeg(P.t), P.t.warp_unit_tasks,
-                P.t.cta_unit_tasks, P.t.slice_max, P.ps.get(), P.pl.get(), P.pz.get(), L.small, L.large, L.zone);
+            k_unit_fill<<<grid_for(P.V, 256, G), 256, 0, st>>>(P.views, P.vpre, P.num, P.V, P.rule, P.ps.get(),
+                                                               P.pl.get(), P.pz.get(), L.small, L.large, L.zone);
         }
         TC_LAUNCH_CHECK();
     }
@@ -1314,9 +1491,9 @@ UnitLists fill_units(UnitPlan& P, int64_t ns, int64_t nl, int64_t nz, Alloc& al,
 }
 
 UnitLists build_unit_lists(const GraphView* views_dev, const int64_t* vpre_dev, int num, int64_t V,
-                           const tc_tuning& t, Alloc& al, cudaStream_t st) {
+                           const UnitRule& rule, Alloc& al, cudaStream_t st) {
     UnitPlan P;
-    plan_units(P, views_dev, vpre_dev, num, V, t, al, st);
+    plan_units(P, views_dev, vpre_dev, num, V, rule, al, st);
     int64_t ns = 0, nl = 0, nz = 0;
     TC_CUDA(cudaMemcpyAsync(&ns, P.ps.get() + V, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     TC_CUDA(cudaMemcpyAsync(&nz, P.pz.get() + V, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
@@ -1348,6 +1525,7 @@ UnitLists units_of(const tc_graph* g) {
     L.nlarge = g->n_large;
     L.nsmall = g->n_small;
     L.nzone = g->n_zone;
+    L.zones = g->zcap > 0;
     return L;
 }
 
@@ -1357,20 +1535,18 @@ size_t count_smem_bytes(bool pv, int threads, int unit_tasks) {
            sizeof(unsigned short) * (size_t)unit_tasks;
 }
 
-using CountKernel = void (*)(const GraphView*, const Unit*, int64_t, const Unit*, int64_t, int, int, int, int,
-                            unsigned*, unsigned long long*);
+using CountKernel = void (*)(const GraphView*, const Unit*, int64_t, const Unit*, int64_t, int, int, unsigned*,
+                            unsigned long long*);
 
-// the count kernel instance for a launch: per-vertex or totals, with or
-// without the search path for short pivot rows, or the instance that counts
-// one tile of a host-resident graph (a window of rows); each in its bucket
-// form for table_mode 1 (the search path is not used there)
-CountKernel count_kernel(bool pv, bool merge, bool win, bool buckets) {
-    if (buckets)
-        return win ? (pv ? k_count<true, false, true, true> : k_count<false, false, true, true>)
-                   : (pv ? k_count<true, false, false, true> : k_count<false, false, false, true>);
-    if (win) return pv ? k_count<true, false, true, false> : k_count<false, false, true, false>;
-    return pv ? (merge ? k_count<true, true, false, false> : k_count<true, false, false, false>)
-              : (merge ? k_count<false, true, false, false> : k_count<false, false, false, false>);
+// the count kernel instance for a launch: per-vertex or totals, the CTA units
+// alone (k_light takes the warps' units), or both in the instance that counts
+// one tile of a host-resident graph (a window of rows) and in the bucket form
+// for table_mode 1
+CountKernel count_kernel(bool pv, bool win, bool buckets) {
+    if (buckets) return win ? (pv ? k_count<true, true, true> : k_count<false, true, true>)
+                            : (pv ? k_count<true, false, true> : k_count<false, false, true>);
+    if (win) return pv ? k_count<true, true, false> : k_count<false, true, false>;
+    return pv ? k_count<true, false, false> : k_count<false, false, false>;
 }
 
 CountLaunch prepare_count(const UnitLists& L, const tc_tuning& t, bool pv, bool win) {
@@ -1379,66 +1555,52 @@ CountLaunch prepare_count(const UnitLists& L, const tc_tuning& t, bool pv, bool 
     c.smem = count_smem_bytes(pv, c.threads, t.cta_unit_tasks);
     c.pv = pv;
     c.buckets = t.table_mode == 1;
-    c.merge = t.merge_max_outdeg > 0 && !win && !c.buckets;
     c.win = win;
-    auto kern = count_kernel(pv, c.merge, c.win, c.buckets);
+    auto kern = count_kernel(pv, c.win, c.buckets);
     TC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.smem));
     int per_sm = 0;
     TC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, c.threads, c.smem));
     per_sm = std::max(per_sm, 1);
     const int64_t warps = (int64_t)num_sms() * per_sm * (c.threads / 32);
     c.grab = L.nsmall < kGrabMin * warps ? 1 : kGrab;
-    const int64_t want =
-        L.nlarge + (L.nsmall + c.grab * (c.threads / 32) - 1) / (c.grab * (c.threads / 32));
+    c.light = !c.win && !c.buckets;
+    const int64_t warp_units = c.light ? 0 : L.nsmall;
+    const int64_t want = L.nlarge + (warp_units + c.grab * (c.threads / 32) - 1) / (c.grab * (c.threads / 32));
+    if (c.light) {
+        TC_CUDA(cudaFuncSetAttribute(pv ? k_light<true> : k_light<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)light_smem(pv)));
+    }
     c.grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)num_sms() * per_sm, want));
     return c;
 }
 
 void launch_count_raw(const CountLaunch& c, const GraphView* views_dev, const UnitLists& L,
-                      const tc_tuning& t, unsigned long long* ctr, cudaStream_t st, unsigned* tlow) {
-    if (L.nlarge + L.nsmall == 0) return;
-    auto kern = count_kernel(c.pv, c.merge, c.win, c.buckets);
-    kern<<<c.grid, c.threads, c.smem, st>>>(views_dev, L.large, L.nlarge, L.small, L.nsmall,
-                                            t.slice_max, t.table_mode, t.merge_max_outdeg, c.grab, tlow, ctr);
-    TC_LAUNCH_CHECK();
+                      const tc_tuning& t, unsigned long long* ctr, cudaStream_t st, unsigned* tlow, bool profile) {
+    if (L.nlarge + (c.light ? 0 : L.nsmall) > 0) {
+        const std::unique_ptr<Prof> prof(profile ? new Prof("k_count", st) : nullptr);
+        auto kern = count_kernel(c.pv, c.win, c.buckets);
+        kern<<<c.grid, c.threads, c.smem, st>>>(views_dev, L.large, L.nlarge, L.small, L.nsmall, t.slice_max, c.grab,
+                                                tlow, ctr);
+        TC_LAUNCH_CHECK();
+    }
+    if (c.light && L.nzone + L.nsmall > 0) {
+        // as many warp units at a time as leave every warp a turn
+        const int64_t warps = (int64_t)num_sms() * kLightMinBlocks * (kMidThreads / 32);
+        const int grab = (int)std::max<int64_t>(1, std::min<int64_t>(kFlatUnits, L.nsmall / warps));
+        const int64_t items = L.nzone + (L.nsmall + grab - 1) / grab;
+        const unsigned blocks = (unsigned)std::min<int64_t>((items + kMidThreads / 32 - 1) / (kMidThreads / 32),
+                                                            (int64_t)num_sms() * kLightMinBlocks);
+        const std::unique_ptr<Prof> prof(profile ? new Prof("k_light", st) : nullptr);
+        auto kern = c.pv ? k_light<true> : k_light<false>;
+        kern<<<blocks, kMidThreads, light_smem(c.pv), st>>>(views_dev, L.zone, L.nzone, L.small, L.nsmall, grab, tlow,
+                                                            ctr);
+        TC_LAUNCH_CHECK();
+    }
 }
 
 void launch_count(const GraphView* views_dev, const UnitLists& L, const tc_tuning& t, bool pv,
                   unsigned long long* ctr, cudaStream_t st, bool profile, unsigned* tlow, bool win) {
-    if (L.nlarge + L.nsmall == 0) return;
-    const CountLaunch c = prepare_count(L, t, pv, win);
-    if (profile) {
-        Prof prof_("k_count", st);
-        launch_count_raw(c, views_dev, L, t, ctr, st, tlow);
-    } else {
-        launch_count_raw(c, views_dev, L, t, ctr, st, tlow);
-    }
-}
-
-void launch_mid(const GraphView* views_dev, const UnitLists& L, const tc_tuning& t, bool pv,
-                unsigned long long* ctr, cudaStream_t st, unsigned* tlow, bool profile) {
-    if (L.nzone == 0 || mid_max_outdeg(t) == 0) return;
-    const size_t smem = sizeof(unsigned) * mid_warp_words(pv) * (kMidThreads / 32);
-    const unsigned blocks = (unsigned)std::min<int64_t>((L.nzone + kMidThreads / 32 - 1) / (kMidThreads / 32),
-                                                        (int64_t)num_sms() * 4);
-    auto go = [&]() {
-        if (pv) k_mid<true><<<blocks, kMidThreads, smem, st>>>(views_dev, L.zone, L.nzone, tlow, ctr);
-        else k_mid<false><<<blocks, kMidThreads, smem, st>>>(views_dev, L.zone, L.nzone, tlow, ctr);
-    };
-    if (profile) {
-        Prof prof_("k_mid", st);
-        go();
-    } else {
-        go();
-    }
-    TC_LAUNCH_CHECK();
-}
-
-void prepare_mid() {
-    TC_CUDA(cudaFuncSetAttribute(k_mid<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(sizeof(unsigned) * mid_warp_words(true) * (kMidThreads / 32))));
-    TC_CUDA(cudaFuncSetAttribute(k_mid<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(sizeof(unsigned) * mid_warp_words(false) * (kMidThreads / 32))));
+    launch_count_raw(prepare_count(L, t, pv, win), views_dev, L, t, ctr, st, tlow, profile);
 }
 
 void build_units(tc_graph* g, const tc_tuning& t, cudaStream_t st) {
@@ -1447,7 +1609,7 @@ void build_units(tc_graph* g, const tc_tuning& t, cudaStream_t st) {
     Buf<int64_t> vpre(al, 2);
     const int64_t hv[2] = {0, g->n};
     TC_CUDA(cudaMemcpyAsync(vpre.get(), hv, sizeof(hv), cudaMemcpyHostToDevice, st));
-    UnitLists L = build_unit_lists(g->view, vpre.get(), 1, g->n, tt, al, st);
+    UnitLists L = build_unit_lists(g->view, vpre.get(), 1, g->n, unit_rule(tt, false, g->zcap > 0), al, st);
     adopt_units(g, L, tt);
 }
 
@@ -1461,8 +1623,6 @@ void count_components(tc_graph* g, const tc_tuning& t, uint64_t* comp_totals_dev
                                      reinterpret_cast<char*>(g->counters)), st));
     const UnitLists L = units_of(g);
     launch_count(g->view_comp, L, tt, false, g->counters, st, true, nullptr);
-    if (L.nzone > 0) prepare_mid();
-    launch_mid(g->view_comp, L, tt, false, g->counters, st, nullptr, true);
     launch_zone(g->view_comp, L, false, g->counters, st, nullptr, true);
     TC_CUDA(cudaMemcpyAsync(comp_totals_dev, g->comp_totals, sizeof(uint64_t) * (size_t)g->num_comps,
                             cudaMemcpyDeviceToDevice, st));
@@ -1488,8 +1648,6 @@ void count(tc_graph* g, const tc_tuning& t, uint64_t* total_dev, uint64_t* per_v
     }
     const UnitLists L = units_of(g);
     launch_count(g->view, L, tt, pv, g->counters, st, true, tlow32 ? g->tlow : nullptr);
-    if (L.nzone > 0) prepare_mid();
-    launch_mid(g->view, L, tt, pv, g->counters, st, tlow32 ? g->tlow : nullptr, true);
     launch_zone(g->view, L, pv, g->counters, st, tlow32 ? g->tlow : nullptr, true);
     if (pv && g->n > 0) {
         {

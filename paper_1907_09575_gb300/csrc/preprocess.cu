@@ -23,7 +23,6 @@
 
 #include "common.cuh"
 #include "tc_internal.cuh"
-#include "zone.cuh"
 
 namespace tc {
 namespace {
@@ -1131,7 +1130,7 @@ void preprocess_with_components(tc_graph* g, const int32_t* src_in, const int32_
     const int64_t hv[2] = {0, n};
     TC_CUDA(cudaMemcpyAsync(gvpre.get(), hv, sizeof(hv), cudaMemcpyHostToDevice, st));
     UnitPlan plan;
-    plan_units(plan, g->view, gvpre.get(), 1, n, def, al, st);
+    plan_units(plan, g->view, gvpre.get(), 1, n, unit_rule(def, false, g->zcap > 0), al, st);
     unsigned long long hprobes[3] = {0, 0, 0};
     int64_t ntasks = 0, ns = 0, nl = 0, nz = 0;
     int herr = 0;

@@ -1,12 +1,12 @@
 // Declarations shared between the preprocessing, counting and API units.
 #pragma once
 #include "common.cuh"
+#include "zone.cuh"
 
 namespace tc {
 
 constexpr int kSmallTable = 128;     // hash slots of a warp unit's table
 constexpr int kSmallMaxOutdeg = 64;  // largest pivot row a warp unit takes
-constexpr int kMidMaxOutdeg = 256;   // largest pivot row counted by one warp, beside the zones
 constexpr int kMaxSlice = 4096;      // largest pivot slice a CTA unit tables
 constexpr int kMaxUnitTasks = 8192;  // 16-bit hit counters; a shared long-task queue
 
@@ -59,7 +59,8 @@ struct UnitLists {
     Unit* large = nullptr;
     Unit* small = nullptr;
     Unit* zone = nullptr;
-    int64_t nlarge = 0, nsmall = 0, nzone = 0;
+    int64_t nlarge = 0, nsmall = 0, nzone = 0;   // zone: pivots of more than kZoneMinPivot entries
+    bool zones = false;   // some graph has dense zones
 };
 
 // Unit building in two phases: plan_units launches the counting kernels and
@@ -72,17 +73,18 @@ struct UnitPlan {
     int num = 0;
     const GraphView* views = nullptr;
     const int64_t* vpre = nullptr;
-    tc_tuning t{};
+    UnitRule rule{};
 };
 void plan_units(UnitPlan& P, const GraphView* views_dev, const int64_t* vpre_dev, int num, int64_t V,
-                const tc_tuning& t, Alloc& al, cudaStream_t st);
+                const UnitRule& rule, Alloc& al, cudaStream_t st);
+UnitRule unit_rule(const tc_tuning& t, bool win, bool zones);
 UnitLists fill_units(UnitPlan& P, int64_t ns, int64_t nl, int64_t nz, Alloc& al, cudaStream_t st);
 UnitLists units_of(const tc_graph* g);
 void adopt_units(tc_graph* g, const UnitLists& L, const tc_tuning& tt);
 
 tc_tuning clamp_tuning(const tc_tuning& t);
 UnitLists build_unit_lists(const GraphView* views_dev, const int64_t* vpre_dev, int num, int64_t V,
-                           const tc_tuning& t, Alloc& al, cudaStream_t st);
+                           const UnitRule& rule, Alloc& al, cudaStream_t st);
 size_t count_smem_bytes(bool pv, int threads, int unit_tasks);
 struct CountLaunch {
     unsigned grid = 1;
@@ -90,7 +92,7 @@ struct CountLaunch {
     size_t smem = 0;
     int grab = 1;         // warp units popped per queue access
     bool pv = false;
-    bool merge = false;   // the instance with the search path for short pivot rows
+    bool light = false;   // k_light takes the warp units and the pivots of up to kMidMaxOutdeg entries
     bool win = false;     // the instance that counts one tile (a window of rows)
     bool buckets = false; // the instance that puts every CTA slice in 4-slot buckets (table_mode 1)
 };
@@ -101,17 +103,12 @@ CountLaunch prepare_count(const UnitLists& L, const tc_tuning& t, bool pv, bool 
 // receive each task's share, or null to add it to the 64-bit accumulator.
 void launch_count_raw(const CountLaunch& c, const GraphView* views_dev, const UnitLists& L,
                       const tc_tuning& t, unsigned long long* ctr, cudaStream_t st,
-                      unsigned* tlow = nullptr);
+                      unsigned* tlow = nullptr, bool profile = false);
 // Launches the count kernel; ctr holds the queue heads and work counters.
 // win: the tile instance, reading the row window (i0, i1, tail_shift) of the view
 void launch_count(const GraphView* views_dev, const UnitLists& L, const tc_tuning& t, bool pv,
                   unsigned long long* ctr, cudaStream_t st, bool profile, unsigned* tlow = nullptr,
                   bool win = false);
-// The pivots that warps count beside the zones (none with buckets everywhere)
-inline int mid_max_outdeg(const tc_tuning& t) { return t.table_mode == 1 ? 0 : kMidMaxOutdeg; }
-void prepare_mid();   // shared-memory attributes: call it outside stream capture
-void launch_mid(const GraphView* views_dev, const UnitLists& L, const tc_tuning& t, bool pv,
-                unsigned long long* ctr, cudaStream_t st, unsigned* tlow, bool profile);
 // Dense zones (zone.cu): the blocks of every row; the zone units' part of a
 // count; the tasks' tails whole again.
 void zone_rows(const tc_graph* g, unsigned* nblocks, cudaStream_t st);

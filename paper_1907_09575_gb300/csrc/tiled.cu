@@ -288,7 +288,7 @@ void count_tiled(const tc_graph* g, int64_t budget, Alloc& al, const tc_tuning& 
         TC_CUDA(cudaMemcpyAsync(view.get(), &v, sizeof(v), cudaMemcpyHostToDevice, st));
         TC_CUDA(cudaMemcpyAsync(vpre.get(), hv, sizeof(hv), cudaMemcpyHostToDevice, st));
         UnitPlan P;
-        plan_units(P, view.get(), vpre.get(), 1, nJ, tt, al, st);
+        plan_units(P, view.get(), vpre.get(), 1, nJ, unit_rule(tt, true, false), al, st);
         int64_t cnt[2] = {0, 0};
         TC_CUDA(cudaMemcpyAsync(&cnt[0], P.ps.get() + nJ, 8, cudaMemcpyDeviceToHost, st));
         TC_CUDA(cudaMemcpyAsync(&cnt[1], P.pl.get() + nJ, 8, cudaMemcpyDeviceToHost, st));

@@ -22,7 +22,6 @@
 
 #include "common.cuh"
 #include "tc_internal.cuh"
-#include "zone.cuh"
 
 namespace tc {
 namespace {
@@ -384,7 +383,7 @@ void zone_restore(const tc_graph* g, cudaStream_t st) {
 
 void launch_zone(const GraphView* views_dev, const UnitLists& L, bool pv, unsigned long long* ctr, cudaStream_t st,
                  unsigned* tlow, bool profile) {
-    if (L.nzone == 0) return;
+    if (L.nzone == 0 || !L.zones) return;
     const unsigned blocks =
         (unsigned)std::min<int64_t>((L.nzone + kZW - 1) / kZW, (int64_t)num_sms() * (pv ? 3 : 4));
     auto go = [&]() {

@@ -33,6 +33,7 @@ constexpr int kZoneMax = (1 << kZoneNzBits) - 1;
 constexpr int kZoneMinCount = TC_ZONE_MIN_COUNT;     // entries of zone 0 ...
 constexpr int kZoneMinCount2 = TC_ZONE_MIN_COUNT2;   // ... and of a further one
 constexpr int kZoneMinRow = 32;
+constexpr int kMidMaxOutdeg = 256;    // largest pivot row that one warp counts
 constexpr int kZoneMinPivot = 64;
 constexpr int kZoneTasks = 248;       // tasks of one unit of the zone kernel: a label's hits fit a byte
 
@@ -106,5 +107,39 @@ __device__ __forceinline__ int zone_cut(uint2 zr, bool big, int64_t e, int len, 
     *z = zr.x;
     return (int)max64((int64_t)zr.y - e - 1, 0);
 }
+
+// ---------------------------------------------------------------------------
+// Which units a pivot of dp entries and nt tasks becomes: `small` ones (flat,
+// k_light's second part), `large` ones (a CTA each) and `wide` ones, which
+// k_light's first part counts with a table per warp (dp <= kMidMaxOutdeg) and
+// the zone kernel visits (more than kZoneMinPivot entries, in a graph with
+// zones; those above kMidMaxOutdeg are large as well).  A pivot of few
+// entries is wide when its tasks make a table worth its building: about
+// 600 instructions against 45 more a warp's step of the flat search.
+#ifndef TC_FLAT_WORK
+#define TC_FLAT_WORK 1024
+#endif
+constexpr int64_t kFlatWork = TC_FLAT_WORK;
+static_assert(kFlatWork / 64 >= 16, "a wide pivot of few entries has at least 16 tasks");
+
+struct UnitRule {
+    int small_max, mid_max;   // mid_max 0: no wide pivots but the zones' own
+    int warp_tasks, cta_tasks, wide_tasks, slice;
+};
+
+__host__ __device__ __forceinline__ void unit_split(const UnitRule& r, bool zoned, int64_t dp, int64_t nt,
+                                                    int64_t& small, int64_t& large, int64_t& wide) {
+    small = large = wide = 0;
+    if (dp <= 0 || nt <= 0) return;
+    const bool mid = dp <= r.mid_max && (dp > kZoneMinPivot || (dp <= r.small_max && dp * nt >= kFlatWork));
+    if (mid || (zoned && dp > kZoneMinPivot)) wide = (nt + r.wide_tasks - 1) / r.wide_tasks;
+    if (mid) return;
+    if (dp <= r.small_max) small = (nt + r.warp_tasks - 1) / r.warp_tasks;
+    else large = ((dp + r.slice - 1) / r.slice) * ((nt + r.cta_tasks - 1) / r.cta_tasks);
+}
+
+// Tasks of a wide unit: what the zone kernel's planes hold, or, in a graph
+// without zones (small: its units hardly fill the SMs), few.
+inline int wide_unit_tasks(bool zones) { return zones ? kZoneTasks : 64; }
 
 }  // namespace tc
