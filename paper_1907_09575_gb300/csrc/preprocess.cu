@@ -7,8 +7,8 @@
 //                     inputs: LSD radix sort, first of each run kept -- the
 //                     set's random atomics into a table of 2^31 slots ran
 //                     slower than the sort's passes (measured at 2^30 pairs).
-//   a3 degrees        d(v) counted when a key enters the set / from the
-//                     unique runs
+//   a3 degrees        d(v) counted when a key enters the set / high ids in the
+//                     middle of the sort, low ids from the unique runs
 //   a4 relabel        rank by (d(v), v): the counting sort of Section 5.3 as
 //                     one stable pass on the degree clipped at 255 (nearly
 //                     every vertex), the vertices at or above it then sorted
@@ -159,29 +159,99 @@ __global__ void k_canon(const int32_t* __restrict__ src, const int32_t* __restri
     }
 }
 
-__global__ void k_unique_flags(const uint64_t* __restrict__ keys, int64_t P, uint64_t sentinel,
-                               int32_t* __restrict__ flags) {
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < P;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        uint64_t k = keys[e];
-        flags[e] = (k != sentinel && (e == 0 || keys[e - 1] != k)) ? 1 : 0;
+// a3, the high ends: keys sorted on the low `sorted` bits of their high id
+// (its `bits` bits are the key's lowest), duplicates among them: each lane's
+// id is counted once per warp and value.  Sorted on all of them, equal ids
+// are neighbours; otherwise at most 2^(bits - sorted) <= 16 values interleave
+// and the lanes of a value find one another.  Counting here, in the middle of
+// the sort, takes an atomic for every few keys; counted in the sorted keys,
+// where the high ids are in no order, every key took its own (2^30 keys: 21
+// ms; the duplicates are taken off again below).
+__global__ void __launch_bounds__(256) k_count_high(const uint64_t* __restrict__ keys, int64_t P, int bits, int sorted,
+                                                    uint64_t sentinel, int32_t* __restrict__ deg) {
+    const uint64_t mask = (1ull << bits) - 1ull;
+    const int lane = threadIdx.x & 31;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t base = blockIdx.x * (int64_t)blockDim.x; base < P; base += 4 * stride) {
+        int32_t v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int64_t e = base + u * stride + threadIdx.x;
+            const uint64_t k = e < P ? keys[e] : sentinel;
+            v[u] = k != sentinel ? (int32_t)(k & mask) : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (sorted == bits) {
+                warp_add_sorted(deg, v[u], v[u] >= 0);
+            } else {
+                const unsigned peers = __match_any_sync(0xffffffffu, v[u]);
+                if (v[u] >= 0 && lane == __ffs(peers) - 1) atomicAdd(&deg[v[u]], __popc(peers));
+            }
+        }
     }
 }
 
-// Adds c to counter[v] once per group of lanes holding the same v.
-__global__ void k_unique_compact(const uint64_t* __restrict__ keys, const int32_t* __restrict__ flags,
-                                 const int64_t* __restrict__ pos, int64_t P, int bits,
-                                 uint64_t* __restrict__ E, int32_t* __restrict__ deg) {
+// a2 + a3 of the sorted keys: the first of each run goes to E and counts in
+// the degree of its low id; the others are taken off the high id's again.
+// A block takes chunks, keeps their keys in order and reserves their place in
+// E with one atomic (E as a whole need not be in order: a5 sorts it).
+constexpr int kUniqueItems = 16;
+__global__ void __launch_bounds__(256) k_unique(const uint64_t* __restrict__ keys, int64_t P, uint64_t sentinel,
+                                                int bits, uint64_t* __restrict__ E,
+                                                unsigned long long* __restrict__ count, int32_t* __restrict__ deg) {
+    __shared__ unsigned part[kUniqueItems * 8];   // kept keys of each row of 32, then those before it
+    __shared__ unsigned long long s_base;
     const uint64_t mask = (1ull << bits) - 1ull;
-    // grid-stride with whole-warp iterations so the warp intrinsics see full warps
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = blockIdx.x * (int64_t)blockDim.x; base < P; base += stride) {
-        int64_t e = base + threadIdx.x;
-        bool keep = e < P && flags[e];
-        uint64_t k = keep ? keys[e] : 0;
-        if (keep) E[pos[e]] = k;
-        warp_add_sorted(deg, (int32_t)(k >> bits), keep);   // keys sorted: min ids in runs
-        if (keep) atomicAdd(&deg[(int32_t)(k & mask)], 1);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t chunk = kUniqueItems * 256;
+    for (int64_t c0 = blockIdx.x * chunk; c0 < P; c0 += gridDim.x * chunk) {
+        uint64_t k[kUniqueItems];
+        unsigned kept[kUniqueItems];
+#pragma unroll
+        for (int u = 0; u < kUniqueItems; ++u) {
+            const int64_t e = c0 + u * 256 + threadIdx.x;
+            k[u] = e < P ? keys[e] : sentinel;
+        }
+#pragma unroll
+        for (int u = 0; u < kUniqueItems; ++u) {
+            const int64_t e = c0 + u * 256 + threadIdx.x;
+            uint64_t before = __shfl_up_sync(0xffffffffu, k[u], 1);
+            if (lane == 0) before = e > 0 && e < P ? keys[e - 1] : ~k[u];
+            const bool edge = k[u] != sentinel, keep = edge && before != k[u];
+            kept[u] = __ballot_sync(0xffffffffu, keep);
+            if (lane == 0) part[u * 8 + w] = __popc(kept[u]);
+            warp_add_sorted(deg, (int32_t)(k[u] >> bits), keep);   // keys sorted: low ids in runs
+            if (edge && !keep) atomicSub(&deg[(int32_t)(k[u] & mask)], 1);
+        }
+        __syncthreads();
+        if (w == 0) {
+            unsigned x[kUniqueItems / 4], sum = 0;
+#pragma unroll
+            for (int q = 0; q < kUniqueItems / 4; ++q) {
+                x[q] = part[lane * (kUniqueItems / 4) + q];
+                sum += x[q];
+            }
+            unsigned inc = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned y = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += y;
+            }
+            unsigned run = inc - sum;
+#pragma unroll
+            for (int q = 0; q < kUniqueItems / 4; ++q) {
+                part[lane * (kUniqueItems / 4) + q] = run;
+                run += x[q];
+            }
+            if (lane == 31) s_base = inc ? atomicAdd(count, (unsigned long long)inc) : 0ull;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < kUniqueItems; ++u)
+            if ((kept[u] >> lane) & 1u)
+                E[s_base + part[u * 8 + w] + __popc(kept[u] & ((1u << lane) - 1u))] = k[u];
+        __syncthreads();   // part and s_base are rewritten by the next chunk
     }
 }
 
@@ -863,24 +933,24 @@ void preprocess_with_components(tc_graph* g, const int32_t* src_in, const int32_
         TC_LAUNCH_CHECK();
         hsrc.release();
         hdst.release();
-        // ids outside [0, n) became sentinels; the error is read at the next sync
-        radix_sort_u64(&keys, &alt, P, 0, 2 * bits, al, st, scal.get());
+        // ids outside [0, n) became sentinels; the error is read at the next
+        // sync.  Sorted first on (whole digits of) the high id, whose degrees
+        // are then counted: no more passes than for all bits at once.
+        const int digits = (bits + 7) / 8;
+        const int high = 2 * digits == (2 * bits + 7) / 8 ? bits : bits / 8 * 8;
+        radix_sort_u64(&keys, &alt, P, 0, high, al, st, scal.get());
         {
-            Buf<int32_t> fl(al, (size_t)P);
-            Buf<int64_t> pos(al, (size_t)P);
-            {
-                Prof prof_("k_unique_flags", st);
-                k_unique_flags<<<grid_for(P, kT, G), kT, 0, st>>>(keys, P, sentinel, fl.get());
-            }
-            TC_LAUNCH_CHECK();
-            exclusive_scan_i32_to_i64(fl.get(), pos.get(), P, tot.get(), al, st);
-            {
-                Prof prof_("k_unique_compact", st);
-                k_unique_compact<<<grid_for(P, kT, G), kT, 0, st>>>(keys, fl.get(), pos.get(), P, bits,
-                                                                alt, deg.get());
-            }
-            TC_LAUNCH_CHECK();
+            Prof prof_("k_count_high", st);
+            k_count_high<<<grid_for(P, kT, G), kT, 0, st>>>(keys, P, bits, high, sentinel, deg.get());
         }
+        TC_LAUNCH_CHECK();
+        radix_sort_u64(&keys, &alt, P, high, 2 * bits, al, st, scal.get());
+        {
+            Prof prof_("k_unique", st);
+            k_unique<<<grid_for(P, kT * kUniqueItems, G), kT, 0, st>>>(
+                keys, P, sentinel, bits, alt, reinterpret_cast<unsigned long long*>(tot.get()), deg.get());
+        }
+        TC_LAUNCH_CHECK();
         std::swap(keys, alt);  // E now in `keys`
     }
     // one synchronisation for: errors so far, m, max degree, heavy vertices
