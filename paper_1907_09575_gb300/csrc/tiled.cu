@@ -32,9 +32,6 @@
 namespace tc {
 namespace {
 
-
-
-
 struct JBlock {
     int64_t j0, j1;   // pivots [j0, j1)
     int64_t t0, t1;   // their tasks [t0, t1) (a sub-range when one pivot is split)
@@ -46,6 +43,37 @@ struct IBlock {
 int64_t off_h(const tc_graph* g, int64_t v) {
     return g->off64 ? static_cast<const int64_t*>(g->host->off)[v]
                     : (int64_t) static_cast<const int32_t*>(g->host->off)[v];
+}
+
+// The offsets of pivots [j0, j0 + count] as the tiles of their block see them
+// -- rows behind capI entries of the row buffer, tasks [t0, t1) of the block --
+// read from the page-locked host arrays where they lie.
+template <class OffT>
+__global__ void k_tile_offsets(const OffT* __restrict__ off, const int64_t* __restrict__ loff, int64_t j0,
+                               int64_t count, int64_t capI, int64_t t0, int64_t t1, int64_t* __restrict__ joff,
+                               int64_t* __restrict__ jloff) {
+    const int64_t c0 = (int64_t)off[j0];
+    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q <= count;
+         q += (int64_t)gridDim.x * blockDim.x) {
+        joff[q] = (int64_t)off[j0 + q] - c0 + capI;
+        jloff[q] = min64(max64(loff[j0 + q], t0), t1) - t0;
+    }
+}
+
+// out[v] = tnew[perm[v]]
+__global__ void k_tile_gather(const uint64_t* __restrict__ tnew, const int32_t* __restrict__ perm, int64_t count,
+                              uint64_t* __restrict__ out) {
+    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < count;
+         v += (int64_t)gridDim.x * blockDim.x)
+        out[v] = tnew[perm[v]];
+}
+
+// device address of page-locked host memory
+template <class T>
+const T* mapped(const T* host) {
+    void* p = nullptr;
+    TC_CUDA(cudaHostGetDevicePointer(&p, const_cast<T*>(host), 0));
+    return static_cast<const T*>(p);
 }
 
 // RAII: a non-blocking stream and events, released on every path
@@ -165,41 +193,38 @@ void count_tiled(const tc_graph* g, int64_t budget, Alloc& al, const tc_tuning& 
                 (long long)maxrow, (long long)budget);
 
     // --- blocks (host, from the host-resident offsets) ----------------------
+    // off and loff only grow, so the end of a block is found by bisection: a
+    // block of several pivots (or rows) ends where any of its limits does.
+    auto upto = [&](int64_t first, auto&& value, int64_t limit) {
+        int64_t lo = first + 1, hi = n;   // largest x in [first + 1, n] with value(x) <= limit (or first + 1)
+        while (lo < hi) {
+            const int64_t mid = (lo + hi + 1) >> 1;
+            if (value(mid) <= limit) lo = mid; else hi = mid - 1;
+        }
+        return lo;
+    };
+    auto row_at = [&](int64_t x) { return off_h(g, x); };
+    auto task_at = [&](int64_t x) { return h->loff[x]; };
     std::vector<JBlock> jb;
     int64_t split_pivots = 0;
     for (int64_t j = 0; j < n;) {
-        const int64_t j0 = j;
-        int64_t rows = 0, tasks = 0;
-        bool split = false;
-        while (j < n) {
-            const int64_t dj = off_h(g, j + 1) - off_h(g, j);
-            const int64_t nt = h->loff[j + 1] - h->loff[j];
-            if (j == j0 && nt > capT) {          // one pivot's tasks over several blocks
-                for (int64_t t = h->loff[j]; t < h->loff[j + 1]; t += capT)
-                    jb.push_back(JBlock{j, j + 1, t, std::min(t + capT, h->loff[j + 1])});
-                ++j;
-                ++split_pivots;
-                split = true;
-                break;
-            }
-            if (j > j0 && (rows + dj > capJ || tasks + nt > capT || j - j0 + 1 > capP)) break;
-            rows += dj;
-            tasks += nt;
+        if (h->loff[j + 1] - h->loff[j] > capT) {   // one pivot's tasks over several blocks
+            for (int64_t t = h->loff[j]; t < h->loff[j + 1]; t += capT)
+                jb.push_back(JBlock{j, j + 1, t, std::min(t + capT, h->loff[j + 1])});
             ++j;
+            ++split_pivots;
+            continue;
         }
-        if (!split && h->loff[j] > h->loff[j0]) jb.push_back(JBlock{j0, j, h->loff[j0], h->loff[j]});
+        const int64_t end = std::min({upto(j, row_at, off_h(g, j) + capJ), upto(j, task_at, h->loff[j] + capT),
+                                      std::max(j + capP, j + 1)});
+        if (h->loff[end] > h->loff[j]) jb.push_back(JBlock{j, end, h->loff[j], h->loff[end]});
+        j = end;
     }
     std::vector<IBlock> ib;
     for (int64_t i = 0; i < n;) {
-        const int64_t i0 = i;
-        int64_t rows = 0;
-        while (i < n) {
-            const int64_t di = off_h(g, i + 1) - off_h(g, i);
-            if (i > i0 && rows + di > capI) break;
-            rows += di;
-            ++i;
-        }
-        ib.push_back(IBlock{i0, i});
+        const int64_t end = upto(i, row_at, off_h(g, i) + capI);
+        ib.push_back(IBlock{i, end});
+        i = end;
     }
     int64_t maxP = 1, maxT = 1;
     for (const JBlock& b : jb) {
@@ -210,7 +235,7 @@ void count_tiled(const tc_graph* g, int64_t budget, Alloc& al, const tc_tuning& 
     // --- device buffers ---------------------------------------------------------
     Buf<unsigned long long> ctr(al, CTR_COUNT);
     Buf<uint64_t> tnew(al, pv ? (size_t)n : 1);
-    Buf<GraphView> view(al, 1);
+    Buf<GraphView> view(al, std::max<size_t>(ib.size(), 1));
     Buf<int64_t> vpre(al, 2);
     Buf<int32_t> rows[2] = {Buf<int32_t>(al, (size_t)(capI + capJ)), Buf<int32_t>(al, (size_t)(capI + capJ))};
     Buf<Task> jtasks(al, (size_t)maxT);
@@ -218,7 +243,6 @@ void count_tiled(const tc_graph* g, int64_t budget, Alloc& al, const tc_tuning& 
     TC_CUDA(cudaMemsetAsync(ctr.get(), 0, sizeof(unsigned long long) * CTR_COUNT, st));
     if (pv) TC_CUDA(cudaMemsetAsync(tnew.get(), 0, sizeof(uint64_t) * (size_t)n, st));
     Streams S;
-    std::vector<int64_t> hj(maxP + 1), hl(maxP + 1);
     int64_t holds[2] = {-1, -1};   // the row block each buffer holds
     if (ts) {
         *ts = TiledStats{};
@@ -262,13 +286,19 @@ void count_tiled(const tc_graph* g, int64_t budget, Alloc& al, const tc_tuning& 
         }
         TC_CUDA(cudaMemcpyAsync(jtasks.get(), h->tasks + b.t0, sizeof(Task) * (size_t)Tb,
                                 cudaMemcpyHostToDevice, st));
-        for (int64_t q = 0; q <= nJ; ++q) {
-            hj[q] = off_h(g, b.j0 + q) - c0 + capI;
-            hl[q] = std::min(std::max(h->loff[b.j0 + q], b.t0), b.t1) - b.t0;
+        {
+            Prof prof_("k_tile_offsets", st);
+            const unsigned blocks = grid_for(nJ + 1, 256, num_sms());
+            if (g->off64)
+                k_tile_offsets<int64_t><<<blocks, 256, 0, st>>>(mapped(static_cast<const int64_t*>(h->off)),
+                                                                mapped(h->loff), b.j0, nJ, capI, b.t0, b.t1,
+                                                                joff.get(), jloff.get());
+            else
+                k_tile_offsets<int32_t><<<blocks, 256, 0, st>>>(mapped(static_cast<const int32_t*>(h->off)),
+                                                                mapped(h->loff), b.j0, nJ, capI, b.t0, b.t1,
+                                                                joff.get(), jloff.get());
         }
-        // pageable sources: staged before the calls return
-        TC_CUDA(cudaMemcpyAsync(joff.get(), hj.data(), 8 * (size_t)(nJ + 1), cudaMemcpyHostToDevice, st));
-        TC_CUDA(cudaMemcpyAsync(jloff.get(), hl.data(), 8 * (size_t)(nJ + 1), cudaMemcpyHostToDevice, st));
+        TC_LAUNCH_CHECK();
         if (ts) ts->h2d_bytes += 4 * (c1 - c0) * 2 + (int64_t)sizeof(Task) * Tb + 16 * (nJ + 1);
         // work units of the whole pivot block, built once; each tile runs
         // them with its row window and skips tasks of other rows
@@ -285,7 +315,28 @@ void count_tiled(const tc_graph* g, int64_t budget, Alloc& al, const tc_tuning& 
         v.i0 = 0;
         v.i1 = 0;
         const int64_t hv[2] = {0, nJ};
-        TC_CUDA(cudaMemcpyAsync(view.get(), &v, sizeof(v), cudaMemcpyHostToDevice, st));
+        // which buffer holds each tile's rows -- already, or after an upload
+        // into the one not holding the rows counted just before -- and the
+        // tiles' views, in one copy
+        std::vector<int> slots(need.size());
+        std::vector<GraphView> hviews(need.size(), v);
+        {
+            int64_t held[2] = {holds[0], holds[1]};
+            for (size_t a = 0; a < need.size(); ++a) {
+                const int64_t blk = need[a];
+                int slot = held[0] == blk ? 0 : held[1] == blk ? 1 : -1;
+                if (slot < 0) slot = (a > 0 && held[0] == need[a - 1]) ? 1 : 0;
+                held[slot] = blk;
+                if (a + 1 < need.size() && held[0] != need[a + 1] && held[1] != need[a + 1]) held[1 - slot] = need[a + 1];
+                slots[a] = slot;
+                hviews[a].adj = rows[slot].get();
+                hviews[a].i0 = (int32_t)ib[blk].i0;
+                hviews[a].i1 = (int32_t)ib[blk].i1;
+                hviews[a].tail_shift = off_h(g, ib[blk].i0);
+            }
+        }
+        TC_CUDA(cudaMemcpyAsync(view.get(), hviews.data(), sizeof(GraphView) * hviews.size(), cudaMemcpyHostToDevice,
+                                st));
         TC_CUDA(cudaMemcpyAsync(vpre.get(), hv, sizeof(hv), cudaMemcpyHostToDevice, st));
         UnitPlan P;
         plan_units(P, view.get(), vpre.get(), 1, nJ, unit_rule(tt, true, false), al, st);
@@ -298,27 +349,18 @@ void count_tiled(const tc_graph* g, int64_t budget, Alloc& al, const tc_tuning& 
         try {
             for (size_t a = 0; a < need.size(); ++a) {
                 const int64_t blk = need[a];
-                int slot = holds[0] == blk ? 0 : holds[1] == blk ? 1 : -1;
-                if (slot < 0) {
-                    // the buffer not holding the row block counted just before
-                    slot = (a > 0 && holds[0] == need[a - 1]) ? 1 : 0;
-                    upload_rows(blk, slot);
-                }
+                const int slot = slots[a];
+                if (holds[slot] != blk) upload_rows(blk, slot);
                 // the next row block goes out while this tile counts
                 if (a + 1 < need.size()) {
                     const int64_t nb = need[a + 1];
                     if (holds[0] != nb && holds[1] != nb) upload_rows(nb, 1 - slot);
                 }
-                v.adj = rows[slot].get();
-                v.i0 = (int32_t)ib[blk].i0;
-                v.i1 = (int32_t)ib[blk].i1;
-                v.tail_shift = off_h(g, ib[blk].i0);
-                TC_CUDA(cudaMemcpyAsync(view.get(), &v, sizeof(v), cudaMemcpyHostToDevice, st));
                 TC_CUDA(cudaStreamWaitEvent(st, S.ready[slot], 0));
                 TC_CUDA(cudaMemsetAsync(ctr.get() + CTR_SMALL_HEAD, 0, 2 * sizeof(unsigned long long), st));
                 if (L.nlarge + L.nsmall > 0) {
                     Prof prof_("k_count", st);
-                    launch_count_raw(launch, view.get(), L, tt, ctr.get(), st, nullptr);
+                    launch_count_raw(launch, view.get() + a, L, tt, ctr.get(), st, nullptr);
                 }
                 TC_CUDA(cudaEventRecord(S.freed[slot], st));
                 if (ts) ts->tiles += 1;
@@ -334,14 +376,27 @@ void count_tiled(const tc_graph* g, int64_t budget, Alloc& al, const tc_tuning& 
     // totals and per-vertex counts back to the host
     unsigned long long tot = 0;
     TC_CUDA(cudaMemcpyAsync(&tot, ctr.get() + CTR_TOTAL, sizeof(tot), cudaMemcpyDeviceToHost, st));
-    std::vector<uint64_t> tn;
     if (pv) {
-        tn.resize((size_t)n);
-        TC_CUDA(cudaMemcpyAsync(tn.data(), tnew.get(), 8 * (size_t)n, cudaMemcpyDeviceToHost, st));
+        // per-vertex counts in original ids: gathered on the device, in pieces
+        // the row buffers' memory holds, the relabelling read where it lies
+        for (auto& r : rows) r.release();
+        jtasks.release();
+        const int64_t piece = std::max<int64_t>(1, std::min<int64_t>(n, capI / 2));   // 8 B each of 2 x 4 capI
+        Buf<uint64_t> out(al, (size_t)piece);
+        const int32_t* perm = mapped(h->perm);
+        for (int64_t v0 = 0; v0 < n; v0 += piece) {
+            const int64_t count = std::min(piece, n - v0);
+            {
+                Prof prof_("k_tile_gather", st);
+                k_tile_gather<<<grid_for(count, 256, num_sms() * 8), 256, 0, st>>>(tnew.get(), perm + v0, count,
+                                                                                  out.get());
+            }
+            TC_LAUNCH_CHECK();
+            TC_CUDA(cudaMemcpyAsync(per_vertex_host + v0, out.get(), 8 * (size_t)count, cudaMemcpyDeviceToHost, st));
+        }
+        out.release();
     }
     TC_CUDA(cudaStreamSynchronize(st));
-    if (pv)
-        for (int64_t v = 0; v < n; ++v) per_vertex_host[v] = tn[(size_t)h->perm[v]];
     *total_host = tot;
     if (ts) {
         unsigned long long c[CTR_COUNT];
