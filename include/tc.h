@@ -77,21 +77,27 @@ typedef struct {
  * depend on the graph's size; tc_tuning_default leaves those at zero).  The
  * count never depends on them; only speed does. */
 typedef struct {
-    int32_t small_max_outdeg;  /* pivots with |U_j| <= this go to warp units (<= 64) */
+    int32_t small_max_outdeg;  /* pivots with |U_j| <= this go to warp units (<= 64): their
+                                  tasks are dealt to the lanes of a warp and each probe
+                                  searches its pivot's sorted row (the list-based
+                                  traversal of Section 3.1), or, with many tasks, the
+                                  pivot gets a table per warp */
     int32_t warp_unit_tasks;   /* tasks per warp unit (<= 8192); 0: 16 for graphs of
                                   fewer than 2^21 edges, else 64 */
     int32_t cta_unit_tasks;    /* tasks per CTA unit (<= 8192) */
-    int32_t cta_threads;       /* threads per CTA of the large-pivot kernel (64..256) */
+    int32_t cta_threads;       /* threads per CTA of the large-pivot kernel (64..256);
+                                  pivots of 65 to 256 entries are counted by single
+                                  warps, which no knob changes */
     int32_t slice_max;         /* pivot entries tabled at once by one CTA (64..4096) */
     int32_t table_mode;        /* 0: a bitmap when the pivot's label span fits (the
                                   direct-index case of Section 5.2), else an exact
                                   tag table (a hash that is a bijection of the
                                   label); 1: the AND-hash of Section 5.2 in 4-slot
                                   buckets for every pivot (the hashed-pivot
-                                  ablation; merge_max_outdeg is then not used) */
-    int32_t merge_max_outdeg;  /* warp-unit pivots with |U_j| <= this build no table:
-                                  each lane searches the sorted row (the list-based
-                                  traversal of Section 3.1); 0 = never (<= 64) */
+                                  ablation; entries in dense zones are tested as
+                                  bits in either mode) */
+    int32_t merge_max_outdeg;  /* accepted (<= 64) and without effect: the rows of
+                                  warp units are searched at any size */
     int32_t reserved;
 } tc_tuning;
 
@@ -104,8 +110,8 @@ typedef struct {
     int64_t max_outdeg;     /* max |U_v| */
     int64_t tasks;          /* edges (i,j) of U with a nonempty part of U_i after j */
     uint64_t probes;        /* sum over tasks of |{k in U_i : k > j}| = sum_i C(|U_i|,2) */
-    int64_t small_units;    /* work units of the warp kernel */
-    int64_t large_units;    /* work units of the CTA kernel */
+    int64_t small_units;    /* work units of pivots searched by warps */
+    int64_t large_units;    /* work units of the CTA kernel (pivots above 256 entries) */
     int64_t device_bytes;   /* bytes held by the graph's arena */
     int32_t offset_bytes;   /* 4 or 8 */
     int32_t pad;
@@ -278,8 +284,9 @@ TC_API tc_status tc_count_tiled(const tc_graph* g, int64_t device_budget_bytes, 
                                 tc_tiled_stats* stats, void* stream);
 
 /* Work done by the last tc_count on a graph, read from device counters:
- * index 0 is the warp kernel (pivots with |U_j| <= small_max_outdeg), index 1
- * the CTA kernel.  probes = entries of the rows U_i read and looked up. */
+ * index 0 is the pivots searched by warps (|U_j| <= small_max_outdeg), index 1
+ * those with a table, of a warp or a CTA.  probes = entries of the rows U_i
+ * looked up, one by one or as bits of a dense zone's block (index 1). */
 typedef struct {
     uint64_t triangles;
     uint64_t units[2];    /* work units processed */
@@ -356,7 +363,7 @@ TC_API tc_status tc_generate_rmat(uint64_t seed, int32_t scale, int64_t n, int64
  * counted by one persistent launch).  A batch references its graphs' arenas:
  * they must stay alive, unchanged, until tc_batch_free.  The batch owns a
  * view table, merged work units over all graphs and a captured CUDA graph
- * (two memsets and the count kernel), replayed by tc_batch_count.
+ * (two memsets and the count kernels), replayed by tc_batch_count.
  *
  * tc_batch_create: graphs = num graph handles (num >= 1); tune NULL for
  *   defaults; stream unused (the batch works on a private stream and
@@ -366,9 +373,8 @@ TC_API tc_status tc_generate_rmat(uint64_t seed, int32_t scale, int64_t n, int64
  *   receives num device uint64 totals, in the order the graphs were given.
  *   Stream ordered; one count at a time per batch.
  * tc_batch_autotune: times candidate tunings (reps replays each: warp/CTA
- *   bin boundary, tasks per warp and per CTA unit, CTA threads, and the
- *   merge threshold below which short pivot rows are searched rather than
- *   tabled) and keeps the fastest; the choice is cached per degree profile (graph count, mean
+ *   bin boundary, tasks per warp and per CTA unit, CTA threads) and keeps the
+ *   fastest; the choice is cached per degree profile (graph count, mean
  *   edges, largest pivot row, mean tail length) for later batches in the
  *   process.  *chosen (may be NULL) receives it.  Synchronises `stream`.
  * tc_batch_get_count_stats: work counters of the last tc_batch_count;

@@ -5,7 +5,7 @@
 // The batch lists its graphs by ascending edge count in a device view table;
 // the unit lists cover all graphs (heaviest pivots of the largest graph
 // first) and each unit adds its hits to its own graph's total.  Counting the
-// batch is one cudaGraphLaunch: two memsets and the count kernel.
+// batch is one cudaGraphLaunch: two memsets and the count kernels.
 #include <algorithm>
 #include <cmath>
 #include <cstring>

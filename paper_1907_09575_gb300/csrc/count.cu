@@ -17,12 +17,16 @@
 // clamps it onto a guard bit that is always clear, a bucket lookup rejects
 // it before reading the table, a tag lookup finds no equal tag.
 //
-// Work: units (graph, pivot, slice of U_j, range of tasks).  Pivots with
-// |U_j| <= 64 become warp units (a private table per warp); larger ones CTA
-// units (a shared table, slices of <= 4096 entries).  One persistent kernel
-// pops CTA units first, heaviest pivots first, then warp units; units may
-// come from many graphs at once (the batched form), each graph reached
-// through a view table.
+// Work: units (graph, pivot, slice of U_j, range of tasks), heaviest pivots
+// first, popped by persistent kernels; units may come from many graphs at once
+// (the batched form), each graph reached through a view table.  Pivots above
+// 256 entries are CTA units (k_count: a shared table, slices of <= 4096
+// entries); k_light counts the others, with a table per warp (65 to 256
+// entries, or few entries and many tasks) or by searching the row; in small
+// graphs that have CTA units k_count takes all, warp units after them.  Tails that
+// lie among the top labels of long rows are counted as bits (zone.cu).  Tiles
+// of host-resident graphs and table_mode 1 take k_count's other instances,
+// where pivots of up to 64 entries are warp units with a private table.
 //
 // Per-vertex counts (t[v] = triangles through v): a task's hits credit i once,
 // per-entry hit counters credit k once per unit, j is credited once per unit.
@@ -903,7 +907,9 @@ __device__ __forceinline__ void cta_unit(const GraphView& G, const Unit& U, int 
 // kTagMaxEntries of them; totals only: the second table alone) | long-task
 // queue (unit_tasks x 16 bit).
 // ---------------------------------------------------------------------------
-template <bool PV, bool WIN, bool BUCKETS>
+// SMALL: the warps' units (pivots of up to 64 entries) as well, each with a
+// table; BUCKETS and WIN instances always take them.
+template <bool PV, bool WIN, bool BUCKETS, bool SMALL>
 __global__ void __launch_bounds__(256, TC_LARGE_MINB)
     k_count(const GraphView* __restrict__ views, const Unit* __restrict__ large, int64_t nlarge,
             const Unit* __restrict__ small, int64_t nsmall, int slice_max, int grab, unsigned* tlow,
@@ -950,12 +956,11 @@ __global__ void __launch_bounds__(256, TC_LARGE_MINB)
     if (lane == 0 && probes) atomicAdd(&ctr[CTR_PROBES + 1], (unsigned long long)probes);
     probes = 0;
 
-    // warp units, each warp on its own slice of the region (k_light's in the
-    // ordinary instance)
+    // warp units, each warp on its own slice of the region
     unsigned* wregion = region + w * kSmallRegionWords;
     unsigned* wcnt = cnt + w * (kSmallTable / 2);
     uint64_t staged = 0;
-    while (WIN || BUCKETS) {
+    while (SMALL) {
         long long u0 = 0;
         if (lane == 0) u0 = (long long)atomicAdd(&ctr[CTR_SMALL_HEAD], (unsigned long long)grab);
         u0 = __shfl_sync(0xffffffffu, u0, 0);
@@ -1423,10 +1428,10 @@ __global__ void k_unit_fill(const GraphView* __restrict__ views, const int64_t* 
 UnitRule unit_rule(const tc_tuning& t, bool win, bool zones) {
     UnitRule r;
     r.small_max = t.small_max_outdeg;
-    r.mid_max = win || t.table_mode == 1 ? 0 : kMidMaxOutdeg;
+    r.mid_max = win || t.table_mode == 1 || !zones ? 0 : kMidMaxOutdeg;
     r.warp_tasks = t.warp_unit_tasks;
     r.cta_tasks = t.cta_unit_tasks;
-    r.wide_tasks = wide_unit_tasks(zones);
+    r.wide_tasks = kZoneTasks;
     r.slice = t.slice_max;
     return r;
 }
@@ -1538,15 +1543,17 @@ size_t count_smem_bytes(bool pv, int threads, int unit_tasks) {
 using CountKernel = void (*)(const GraphView*, const Unit*, int64_t, const Unit*, int64_t, int, int, unsigned*,
                             unsigned long long*);
 
-// the count kernel instance for a launch: per-vertex or totals, the CTA units
-// alone (k_light takes the warps' units), or both in the instance that counts
-// one tile of a host-resident graph (a window of rows) and in the bucket form
-// for table_mode 1
-CountKernel count_kernel(bool pv, bool win, bool buckets) {
-    if (buckets) return win ? (pv ? k_count<true, true, true> : k_count<false, true, true>)
-                            : (pv ? k_count<true, false, true> : k_count<false, false, true>);
-    if (win) return pv ? k_count<true, true, false> : k_count<false, true, false>;
-    return pv ? k_count<true, false, false> : k_count<false, false, false>;
+// the count kernel instance for a launch: per-vertex or totals; the CTA units
+// alone (k_light takes the rest), or the warps' units as well: in graphs
+// without zones that have CTA units, in the instance that counts one tile of
+// a host-resident graph (a window of rows) and in the bucket form for
+// table_mode 1
+CountKernel count_kernel(bool pv, bool win, bool buckets, bool small) {
+    if (buckets) return win ? (pv ? k_count<true, true, true, true> : k_count<false, true, true, true>)
+                            : (pv ? k_count<true, false, true, true> : k_count<false, false, true, true>);
+    if (win) return pv ? k_count<true, true, false, true> : k_count<false, true, false, true>;
+    if (small) return pv ? k_count<true, false, false, true> : k_count<false, false, false, true>;
+    return pv ? k_count<true, false, false, false> : k_count<false, false, false, false>;
 }
 
 CountLaunch prepare_count(const UnitLists& L, const tc_tuning& t, bool pv, bool win) {
@@ -1556,14 +1563,15 @@ CountLaunch prepare_count(const UnitLists& L, const tc_tuning& t, bool pv, bool 
     c.pv = pv;
     c.buckets = t.table_mode == 1;
     c.win = win;
-    auto kern = count_kernel(pv, c.win, c.buckets);
+    // a graph with CTA units but no wide ones is small: one kernel for all
+    c.light = !c.win && !c.buckets && (L.nzone > 0 || L.nlarge == 0);
+    auto kern = count_kernel(pv, c.win, c.buckets, !c.light);
     TC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.smem));
     int per_sm = 0;
     TC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, c.threads, c.smem));
     per_sm = std::max(per_sm, 1);
     const int64_t warps = (int64_t)num_sms() * per_sm * (c.threads / 32);
     c.grab = L.nsmall < kGrabMin * warps ? 1 : kGrab;
-    c.light = !c.win && !c.buckets;
     const int64_t warp_units = c.light ? 0 : L.nsmall;
     const int64_t want = L.nlarge + (warp_units + c.grab * (c.threads / 32) - 1) / (c.grab * (c.threads / 32));
     if (c.light) {
@@ -1578,7 +1586,7 @@ void launch_count_raw(const CountLaunch& c, const GraphView* views_dev, const Un
                       const tc_tuning& t, unsigned long long* ctr, cudaStream_t st, unsigned* tlow, bool profile) {
     if (L.nlarge + (c.light ? 0 : L.nsmall) > 0) {
         const std::unique_ptr<Prof> prof(profile ? new Prof("k_count", st) : nullptr);
-        auto kern = count_kernel(c.pv, c.win, c.buckets);
+        auto kern = count_kernel(c.pv, c.win, c.buckets, !c.light);
         kern<<<c.grid, c.threads, c.smem, st>>>(views_dev, L.large, L.nlarge, L.small, L.nsmall, t.slice_max, c.grab,
                                                 tlow, ctr);
         TC_LAUNCH_CHECK();

@@ -553,14 +553,22 @@ __global__ void k_task_count_last(const OffT* __restrict__ off, const int32_t* _
                                   int64_t n, int32_t* __restrict__ tcount,
                                   unsigned long long* __restrict__ probes) {
     unsigned long long my = 0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t re = (int64_t)off[i + 1];
-        const int64_t d = re - (int64_t)off[i];
-        if (d > 0) {
-            atomicSub(&tcount[adj[re - 1]], 1);
-            my += (unsigned long long)(d * (d - 1) / 2);
+    const int lane = threadIdx.x & 31;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t base = blockIdx.x * (int64_t)blockDim.x; base < n; base += stride) {
+        const int64_t i = base + threadIdx.x;
+        int32_t last = -1;
+        if (i < n) {
+            const int64_t re = (int64_t)off[i + 1];
+            const int64_t d = re - (int64_t)off[i];
+            if (d > 0) {
+                last = adj[re - 1];
+                my += (unsigned long long)(d * (d - 1) / 2);
+            }
         }
+        // most rows end at one of few hubs: an atomic a warp and label
+        const unsigned peers = __match_any_sync(0xffffffffu, last);
+        if (last >= 0 && lane == __ffs(peers) - 1) atomicSub(&tcount[last], __popc(peers));
     }
 #pragma unroll
     for (int o = 16; o; o >>= 1) my += __shfl_xor_sync(0xffffffffu, my, o);

@@ -39,10 +39,12 @@ constexpr int kZoneTasks = 248;       // tasks of one unit of the zone kernel: a
 
 // Block capacity of a graph of up to m edges: 2 B an edge (measured need: 0.6
 // B an edge on a Chung-Lu graph to 1.3 B on RMAT scale 20); block 0 stands
-// for none.  No zones up to 2^18 edges: there the two further launches cost
-// what they save or more (RMAT scale 14, 2^18 pairs: step 217 us without
-// zones, 241 us with them; scale 18: count 636 us without, 480 us with).
-inline int64_t zone_capacity(int64_t m) { return m <= (1ll << 18) ? 0 : m / 128; }   // x 256 B: below 2^32
+// for none.  No zones, and no pivots of more than 64 entries for single warps,
+// up to 2^19 edges: there a count is as long as its longest unit, which eight
+// warps share, and the further launches cost what they save (kept RMAT graphs,
+// totals: 2^17 pairs 45 us as CTA units, 60 by warps; 2^18 65 and 75; 2^19 81
+// and 96 with zones; 2^20 132 and 110).
+inline int64_t zone_capacity(int64_t m) { return m <= (1ll << 19) ? 0 : m / 128; }   // x 256 B: below 2^32
 
 // One warp makes the blocks of row r: adj[rb, rb + d), sorted, d >
 // kZoneMinRow.  buf: kZoneWords words of the warp's shared memory.  nblocks
@@ -137,9 +139,5 @@ __host__ __device__ __forceinline__ void unit_split(const UnitRule& r, bool zone
     if (dp <= r.small_max) small = (nt + r.warp_tasks - 1) / r.warp_tasks;
     else large = ((dp + r.slice - 1) / r.slice) * ((nt + r.cta_tasks - 1) / r.cta_tasks);
 }
-
-// Tasks of a wide unit: what the zone kernel's planes hold, or, in a graph
-// without zones (small: its units hardly fill the SMs), few.
-inline int wide_unit_tasks(bool zones) { return zones ? kZoneTasks : 64; }
 
 }  // namespace tc
