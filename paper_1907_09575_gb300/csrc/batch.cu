@@ -60,11 +60,14 @@ void set_tuning(tc_batch* b, const tc_tuning& t) {
         b->units = UnitLists{};
     }
     b->alloc.stream = b->cap;
-    // few tasks a wide unit only while all of the batch's are few
-    b->units = build_unit_lists(b->views, b->vpre, b->num, b->V, unit_rule(tt, false, zone_capacity(m) > 0), b->alloc,
+    // pivots of 65 to 256 entries go to single warps when some graph has zones
+    // (its zone units must not be CTA units too), or the batch its edges
+    bool zones = false;
+    for (const tc_graph* g : b->graphs) zones |= g->zcap > 0;
+    b->units = build_unit_lists(b->views, b->vpre, b->num, b->V, unit_rule(tt, false, zones || zones_at(m)), b->alloc,
                                 b->cap);
     TC_CUDA(cudaStreamSynchronize(b->cap));
-    for (const tc_graph* g : b->graphs) b->units.zones |= g->zcap > 0;
+    b->units.zones = zones;
     b->tuning = tt;
     const CountLaunch c = prepare_count(b->units, tt, false);
     TC_CUDA(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));

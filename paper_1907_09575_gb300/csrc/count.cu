@@ -1235,7 +1235,7 @@ static_assert(sizeof(FlatWarp) <= sizeof(unsigned) * (64 + kMidSlots + kMidSlots
 template <bool PV>
 __global__ void __launch_bounds__(kMidThreads, kLightMinBlocks)
     k_light(const GraphView* __restrict__ views, const Unit* __restrict__ units, int64_t nunits,
-            const Unit* __restrict__ small, int64_t nsmall, int grab, unsigned* tlow,
+            int mid_max, const Unit* __restrict__ small, int64_t nsmall, int grab, unsigned* tlow,
             unsigned long long* __restrict__ ctr) {
     extern __shared__ __align__(16) unsigned smem[];
     __shared__ unsigned long long s_work[kMidThreads / 32][4];
@@ -1258,7 +1258,7 @@ __global__ void __launch_bounds__(kMidThreads, kLightMinBlocks)
         const GraphView G = views[U.g];
         const int64_t rb = off_at(G, U.j);
         const int64_t d = off_at(G, U.j + 1) - rb;
-        if (d > kMidEntries) continue;   // a CTA unit
+        if (d > mid_max) continue;   // a CTA unit
         const int dp = (int)d;
         acc.to(unit_target(G, U));
         const int lo = G.adj[rb], hi = G.adj[rb + dp - 1];
@@ -1478,6 +1478,7 @@ UnitLists fill_units(UnitPlan& P, int64_t ns, int64_t nl, int64_t nz, Alloc& al,
     L.nlarge = nl;
     L.nsmall = ns;
     L.nzone = nz;
+    L.mid_max = P.rule.mid_max;
     if (P.V > 0) {
         {
             Prof prof_("k_unit_fill", st);
@@ -1531,6 +1532,7 @@ UnitLists units_of(const tc_graph* g) {
     L.nsmall = g->n_small;
     L.nzone = g->n_zone;
     L.zones = g->zcap > 0;
+    L.mid_max = unit_rule(g->units_tuning, false, L.zones).mid_max;
     return L;
 }
 
@@ -1600,8 +1602,8 @@ void launch_count_raw(const CountLaunch& c, const GraphView* views_dev, const Un
                                                             (int64_t)num_sms() * kLightMinBlocks);
         const std::unique_ptr<Prof> prof(profile ? new Prof("k_light", st) : nullptr);
         auto kern = c.pv ? k_light<true> : k_light<false>;
-        kern<<<blocks, kMidThreads, light_smem(c.pv), st>>>(views_dev, L.zone, L.nzone, L.small, L.nsmall, grab, tlow,
-                                                            ctr);
+        kern<<<blocks, kMidThreads, light_smem(c.pv), st>>>(views_dev, L.zone, L.nzone, L.mid_max, L.small, L.nsmall,
+                                                            grab, tlow, ctr);
         TC_LAUNCH_CHECK();
     }
 }

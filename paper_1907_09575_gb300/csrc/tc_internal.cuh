@@ -61,6 +61,7 @@ struct UnitLists {
     Unit* zone = nullptr;
     int64_t nlarge = 0, nsmall = 0, nzone = 0;   // zone: pivots of more than kZoneMinPivot entries
     bool zones = false;   // some graph has dense zones
+    int mid_max = 0;      // of the rule: larger pivots of the zone list are CTA units as well
 };
 
 // Unit building in two phases: plan_units launches the counting kernels and

@@ -44,7 +44,10 @@ constexpr int kZoneTasks = 248;       // tasks of one unit of the zone kernel: a
 // warps share, and the further launches cost what they save (kept RMAT graphs,
 // totals: 2^17 pairs 45 us as CTA units, 60 by warps; 2^18 65 and 75; 2^19 81
 // and 96 with zones; 2^20 132 and 110).
-inline int64_t zone_capacity(int64_t m) { return m <= (1ll << 19) ? 0 : m / 128; }   // x 256 B: below 2^32
+// A graph preprocessed in one launch has them by its pairs, which the host
+// knows before its edges: zcap, not m, says whether a graph has zones.
+inline bool zones_at(int64_t m) { return m > (1ll << 19); }
+inline int64_t zone_capacity(int64_t m) { return zones_at(m) ? m / 128 : 0; }   // x 256 B: below 2^32
 
 // One warp makes the blocks of row r: adj[rb, rb + d), sorted, d >
 // kZoneMinRow.  buf: kZoneWords words of the warp's shared memory.  nblocks
