@@ -1041,6 +1041,7 @@ void build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64_t P,
         read_tally();
         cap_m = (int64_t)h.m;
     }
+    g->plan_m = cap_m;
     const tc_tuning tt = clamp_tuning(size_tuning(def, cap_m));
     graph_arena(g, cap_m, off64, num_comps);
     a.off = g->off;

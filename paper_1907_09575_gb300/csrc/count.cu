@@ -1625,7 +1625,7 @@ void build_units(tc_graph* g, const tc_tuning& t, cudaStream_t st) {
 
 void count_components(tc_graph* g, const tc_tuning& t, uint64_t* comp_totals_dev,
                       cudaStream_t st) {
-    const tc_tuning tt = clamp_tuning(size_tuning(t, g->m));
+    const tc_tuning tt = clamp_tuning(size_tuning(t, g->plan_m));
     if (!tuning_equal(tt, g->units_tuning)) build_units(g, tt, st);
     // counters and component totals lie next to each other
     TC_CUDA(cudaMemsetAsync(g->counters, 0,
@@ -1641,7 +1641,7 @@ void count_components(tc_graph* g, const tc_tuning& t, uint64_t* comp_totals_dev
 void count(tc_graph* g, const tc_tuning& t, uint64_t* total_dev, uint64_t* per_vertex_dev,
            cudaStream_t st) {
     // the unit lists are a cache of the tuning they were built for
-    const tc_tuning tt = clamp_tuning(size_tuning(t, g->m));
+    const tc_tuning tt = clamp_tuning(size_tuning(t, g->plan_m));
     if (!tuning_equal(tt, g->units_tuning)) build_units(g, tt, st);
     const bool pv = per_vertex_dev != nullptr;
     // the counters, and with per-vertex counts the accumulators behind them

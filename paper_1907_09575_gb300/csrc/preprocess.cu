@@ -1203,6 +1203,7 @@ void preprocess_with_components(tc_graph* g, const int32_t* src_in, const int32_
     // as the task statistics
     tc_tuning def;
     tuning_defaults(&def);
+    g->plan_m = m;
     def = clamp_tuning(size_tuning(def, m));
     Buf<int64_t> gvpre(al, 2);
     const int64_t hv[2] = {0, n};

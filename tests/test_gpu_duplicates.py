@@ -64,3 +64,26 @@ def test_batch(tc, members, tuning):
     b.free()
     for g in graphs:
         g.free()
+
+
+@pytest.mark.parametrize("pairs", [(1 << 21) - 1, 1 << 21, 1 << 22, (1 << 22) + 1])
+@pytest.mark.parametrize("components", [False, True])
+def test_units_are_planned_once(tc, pairs, components):
+    """The units preprocessing built are those the first default count asks
+    for, whatever share of the pairs are edges."""
+    n = 1 << 15
+    rng = np.random.default_rng(pairs)
+    s, d = (torch.from_numpy(rng.integers(0, n // 8, pairs).astype(np.int32)).cuda() for _ in range(2))
+    s[: pairs // 2], d[: pairs // 2] = s[pairs // 2: 2 * (pairs // 2)].clone(), d[pairs // 2: 2 * (pairs // 2)].clone()
+    g = tc.preprocess_components(s, d, [0, n // 2, n]) if components else tc.preprocess(s, d, n)
+    assert g.stats()["m"] < 1 << 21
+    torch.cuda.synchronize()
+    tc.profile_enable()
+    got = int(tc.count_components(g).sum()) if components else g.count()
+    launched = tc.profile_read()
+    tc.profile_enable(False)
+    assert "k_unit_fill" not in launched, launched
+    t = tc.tuning_default()
+    t.warp_unit_tasks = 5
+    assert g.count(tuning=t) == got
+    g.free()
