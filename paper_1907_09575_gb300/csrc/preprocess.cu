@@ -166,23 +166,41 @@ __global__ void k_canon(const int32_t* __restrict__ src, const int32_t* __restri
 // and the lanes of a value find one another.  Counting here, in the middle of
 // the sort, takes an atomic for every few keys; counted in the sorted keys,
 // where the high ids are in no order, every key took its own (2^30 keys: 21
-// ms; the duplicates are taken off again below).
+// ms; the duplicates are taken off again below).  A warp takes one stretch of
+// neighbouring keys and counts rows of one id together: a counter serves its
+// atomics one after the other, some 20 ns each, and a hub's, or that of a pair
+// given very often, would get one a row (2^27 pairs among 16 vertices: 5.7 ms,
+// 0.19 together; 2^30 RMAT pairs alike).
 __global__ void __launch_bounds__(256) k_count_high(const uint64_t* __restrict__ keys, int64_t P, int bits, int sorted,
                                                     uint64_t sentinel, int32_t* __restrict__ deg) {
     const uint64_t mask = (1ull << bits) - 1ull;
     const int lane = threadIdx.x & 31;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = blockIdx.x * (int64_t)blockDim.x; base < P; base += 4 * stride) {
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    const int64_t stretch = (P + 128 * warps - 1) / (128 * warps) * 128;
+    const int64_t e0 = (blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5)) * stretch;
+    const int64_t e1 = min64(e0 + stretch, P);
+    int32_t of = -1;   // the id of the rows counted together, and their keys
+    int rows = 0;
+    for (int64_t r = e0; r < e1; r += 128) {
         int32_t v[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const int64_t e = base + u * stride + threadIdx.x;
-            const uint64_t k = e < P ? keys[e] : sentinel;
+            const int64_t e = r + 32 * u + lane;
+            const uint64_t k = e < e1 ? keys[e] : sentinel;
             v[u] = k != sentinel ? (int32_t)(k & mask) : -1;
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            if (sorted == bits) {
+            const unsigned on = __ballot_sync(0xffffffffu, v[u] >= 0);   // self-loops lie among the last id's
+            const int32_t v0 = __shfl_sync(0xffffffffu, v[u], __ffs(on | 0x80000000u) - 1);
+            if (__all_sync(0xffffffffu, v[u] == v0 || v[u] < 0)) {
+                if (v0 != of) {
+                    if (lane == 0 && of >= 0) atomicAdd(&deg[of], rows);
+                    of = v0;
+                    rows = 0;
+                }
+                rows += __popc(on);
+            } else if (sorted == bits) {
                 warp_add_sorted(deg, v[u], v[u] >= 0);
             } else {
                 const unsigned peers = __match_any_sync(0xffffffffu, v[u]);
@@ -190,10 +208,13 @@ __global__ void __launch_bounds__(256) k_count_high(const uint64_t* __restrict__
             }
         }
     }
+    if (lane == 0 && of >= 0) atomicAdd(&deg[of], rows);
 }
 
 // a2 + a3 of the sorted keys: the first of each run goes to E and counts in
-// the degree of its low id; the others are taken off the high id's again.
+// the degree of its low id; the others are taken off the high id's again (an
+// atomic each, on one counter where one pair was given 2^27 times, made its
+// preprocessing 90 ms; a run of them at a time 2.7).
 // A block takes chunks, keeps their keys in order and reserves their place in
 // E with one atomic (E as a whole need not be in order: a5 sorts it).
 constexpr int kUniqueItems = 16;
@@ -206,8 +227,8 @@ __global__ void __launch_bounds__(256) k_unique(const uint64_t* __restrict__ key
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t chunk = kUniqueItems * 256;
     for (int64_t c0 = blockIdx.x * chunk; c0 < P; c0 += gridDim.x * chunk) {
-        uint64_t k[kUniqueItems];
-        unsigned kept[kUniqueItems];
+        uint64_t k[kUniqueItems], often = sentinel;
+        unsigned kept[kUniqueItems], more = 0;
 #pragma unroll
         for (int u = 0; u < kUniqueItems; ++u) {
             const int64_t e = c0 + u * 256 + threadIdx.x;
@@ -222,8 +243,19 @@ __global__ void __launch_bounds__(256) k_unique(const uint64_t* __restrict__ key
             kept[u] = __ballot_sync(0xffffffffu, keep);
             if (lane == 0) part[u * 8 + w] = __popc(kept[u]);
             warp_add_sorted(deg, (int32_t)(k[u] >> bits), keep);   // keys sorted: low ids in runs
-            if (edge && !keep) atomicSub(&deg[(int32_t)(k[u] & mask)], 1);
+            // neighbouring duplicates are of one key: an atomic a run, and for
+            // rows of nothing else one for all of them
+            const unsigned dup = __ballot_sync(0xffffffffu, edge && !keep);
+            if (dup == 0xffffffffu) {
+                if (k[u] != often && more && lane == 0) atomicSub(&deg[(int32_t)(often & mask)], (int)more);
+                more = (k[u] != often ? 0 : more) + 32;
+                often = k[u];
+            } else if (edge && !keep && !((dup << 1 >> lane) & 1u)) {
+                const unsigned run = dup >> lane;
+                atomicSub(&deg[(int32_t)(k[u] & mask)], __popc(run & ~(run + 1)));
+            }
         }
+        if (more && lane == 0) atomicSub(&deg[(int32_t)(often & mask)], (int)more);
         __syncthreads();
         if (w == 0) {
             unsigned x[kUniqueItems / 4], sum = 0;
@@ -944,8 +976,10 @@ void preprocess_with_components(tc_graph* g, const int32_t* src_in, const int32_
         // ids outside [0, n) became sentinels; the error is read at the next
         // sync.  Sorted first on (whole digits of) the high id, whose degrees
         // are then counted: no more passes than for all bits at once.
+        // (A graph of up to 16 vertices takes the one more: its few counters
+        // would get an atomic a warp and vertex.)
         const int digits = (bits + 7) / 8;
-        const int high = 2 * digits == (2 * bits + 7) / 8 ? bits : bits / 8 * 8;
+        const int high = bits <= 4 || 2 * digits == (2 * bits + 7) / 8 ? bits : bits / 8 * 8;
         radix_sort_u64(&keys, &alt, P, 0, high, al, st, scal.get());
         {
             Prof prof_("k_count_high", st);

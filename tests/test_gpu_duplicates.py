@@ -87,3 +87,55 @@ def test_units_are_planned_once(tc, pairs, components):
     t.warp_unit_tasks = 5
     assert g.count(tuning=t) == got
     g.free()
+
+
+def build_ms(tc, s, d, n):
+    best = 1e9
+    for _ in range(3):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        tc.preprocess(s, d, n).free()
+        b.record()
+        torch.cuda.synchronize()
+        best = min(best, a.elapsed_time(b))
+    return best
+
+
+@pytest.mark.parametrize("shape", ["one pair", "16 vertices", "hub", "blocks", "shuffled"])
+def test_large_inputs_of_few_edges(tc, shape):
+    """More than 2^26 pairs (the sorted path) with few distinct ones: the graph
+    is that of the distinct pairs, and one counter's share of the duplicates
+    does not hold up the rest."""
+    pairs = (1 << 26) + 77
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    at = torch.arange(pairs, device="cuda")
+    if shape == "one pair":
+        hs, hd, n = np.array([3], np.int32), np.array([7], np.int32), 10
+    elif shape == "16 vertices":
+        i, j = np.triu_indices(16, 1)
+        hs, hd, n = i.astype(np.int32), j.astype(np.int32), 16
+    elif shape == "hub":                      # every edge's larger id is the hub's
+        hs, n = np.arange(4000, dtype=np.int32), 4001
+        hd = np.full(4000, 4000, np.int32)
+    else:
+        hs, hd = inputs.rmat(7, 14, 100_000)
+        n = 1 << 14
+    if shape == "blocks":                     # each pair's copies beside one another
+        pick = at * hs.size // pairs
+    else:
+        pick = torch.randint(0, hs.size, (pairs,), generator=gen, device="cuda")
+        pick[: hs.size] = torch.arange(hs.size, device="cuda")
+    s, d = (torch.from_numpy(x).cuda()[pick] for x in (hs, hd))
+    del pick
+    swap = (at & 1).bool()
+    s, d = torch.where(swap, s, d), torch.where(swap, d, s)
+    del at, swap
+    want, want_t, facts = oracle.count(hs, hd, n, per_vertex=True, stats=True)
+    g = tc.preprocess(s, d, n)
+    total, t = g.count(per_vertex=True)
+    assert total == want and np.array_equal(t.cpu().numpy().astype(np.uint64), want_t)
+    assert (g.stats()["m"], g.stats()["max_deg"]) == (facts["m"], facts["max_deg"])
+    g.free()
+    mine = build_ms(tc, s, d, n)
+    s, d = (torch.randint(0, 1 << 20, (pairs,), generator=gen, dtype=torch.int32, device="cuda") for _ in range(2))
+    assert mine < 2 * build_ms(tc, s, d, 1 << 20)
