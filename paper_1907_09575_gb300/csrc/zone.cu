@@ -326,12 +326,17 @@ __global__ void __launch_bounds__(256) k_zone_rows(const OffT* __restrict__ off,
                                                    uint32_t* zowner, int64_t cap, unsigned* nblocks) {
     __shared__ __align__(8) uint32_t buf[8][kZoneWords];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    // 32 neighbouring rows a warp at a time, fewer where that leaves warps
+    // without: a dense graph has few rows, all of them long (K_8000: 5.8 ms with
+    // 32 a warp, 0.25)
     const int64_t warps = (int64_t)gridDim.x * 8;
-    for (int64_t r0 = ((int64_t)blockIdx.x * 8 + w) * 32; r0 < n; r0 += warps * 32) {
+    int per = 32;
+    while (per > 1 && n < 2 * per * warps) per >>= 1;
+    for (int64_t r0 = ((int64_t)blockIdx.x * 8 + w) * per; r0 < n; r0 += warps * per) {
         const int64_t r = r0 + lane;
         int64_t rb = 0;
         int d = 0;
-        if (r < n) {
+        if (lane < per && r < n) {
             rb = (int64_t)off[r];
             d = (int)((int64_t)off[r + 1] - rb);
             zrow[r] = make_uint2(0, 0);

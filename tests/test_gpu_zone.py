@@ -83,3 +83,22 @@ def test_components(tc):
     got = tc.count_components(g).tolist()
     assert got == [oracle.count(p[0].astype(np.int32), p[1].astype(np.int32), p[2]) for p in parts]
     g.free()
+
+
+@pytest.mark.parametrize("k", [5795, 6001])
+def test_dense_graph_beyond_the_persistent_form(tc, k):
+    """K_k of more than 2^24 pairs: few rows, nearly all of them in several
+    zones; making their blocks takes less than the deduplication."""
+    i, j = torch.triu_indices(k, k, 1, device="cuda")
+    p = torch.randperm(i.numel(), generator=torch.Generator().manual_seed(k)).cuda()
+    s, d = (x[p].to(torch.int32) for x in (i, j))
+    assert s.numel() > 1 << 24
+    tc.preprocess(s, d, k).free()
+    tc.profile_enable()
+    g = tc.preprocess(s, d, k)
+    times = tc.profile_read()
+    tc.profile_enable(False)
+    assert times["k_zone_rows"][1] < 0.5 * times["k_dedup_insert"][1], times
+    total, t = g.count(per_vertex=True)
+    assert total == k * (k - 1) * (k - 2) // 6 and bool((t == (k - 1) * (k - 2) // 2).all())
+    g.free()
