@@ -94,8 +94,7 @@ typedef struct {
                                   tag table (a hash that is a bijection of the
                                   label); 1: the AND-hash of Section 5.2 in 4-slot
                                   buckets for every pivot (the hashed-pivot
-                                  ablation; entries in dense zones are tested as
-                                  bits in either mode) */
+                                  ablation: no bitmaps, no dense zones) */
     int32_t merge_max_outdeg;  /* accepted (<= 64) and without effect: the rows of
                                   warp units are searched at any size */
     int32_t reserved;

@@ -453,7 +453,7 @@ tc_status tc_count_get_stats(const tc_graph* g, tc_count_stats* out, void* strea
         out->probes[k] = c[CTR_PROBES + k];
         out->staged[k] = c[CTR_STAGED + k];
     }
-    out->probes[1] += g->covered;   // entries counted as zone bits
+    out->probes[1] += g->zone_probes;
     TC_API_END
 }
 

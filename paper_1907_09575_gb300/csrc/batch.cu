@@ -300,7 +300,8 @@ tc_status tc_batch_get_count_stats(const tc_batch* b, tc_count_stats* out, void*
     TC_CUDA(cudaStreamSynchronize(st));
     out->triangles = std::accumulate(tot.begin(), tot.end(), (uint64_t)0);
     uint64_t covered = 0;   // entries counted as zone bits
-    for (const tc_graph* g : b->graphs) covered += g->covered;
+    if (b->units.nzone > 0)
+        for (const tc_graph* g : b->graphs) covered += g->covered;
     for (int k = 0; k < 2; ++k) {
         out->units[k] = c[CTR_UNITS + k];
         out->tasks[k] = c[CTR_TASKS + k];

@@ -180,6 +180,7 @@ struct tc_graph {
     struct Unit* zone_units = nullptr;
     int64_t n_zone = 0;
     uint64_t covered = 0;       // tail entries the zones hold, of pivots that use them
+    uint64_t zone_probes = 0;   // of them, those the last count tested there
 
     size_t zero_bytes = 0;      // [counters | comp_totals | tnew | tlow (small graphs)] are one range
     bool tlow_in_arena = false;

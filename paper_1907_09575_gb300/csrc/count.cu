@@ -428,6 +428,18 @@ __device__ __forceinline__ void credit_task(unsigned long long* tnew, unsigned* 
         atomicAdd(&tnew[i], (unsigned long long)c);
 }
 
+__device__ __forceinline__ int64_t off_at(const GraphView& G, int64_t v) {
+    return G.off64 ? static_cast<const int64_t*>(G.off)[v]
+                   : (int64_t) static_cast<const int32_t*>(G.off)[v];
+}
+
+// WHOLE: the length of a task's tail with what the zones hold of it
+template <bool WHOLE>
+__device__ __forceinline__ int tail_length(const GraphView& G, const Task& t) {
+    if (WHOLE && t.zone) return (int)(off_at(G, (int64_t)t.i + 1) - (int64_t)t.start);
+    return t.len;
+}
+
 // ---------------------------------------------------------------------------
 // One warp takes up to 32 tasks [tb, min(tb+32, t1)).
 //
@@ -444,8 +456,8 @@ __device__ __forceinline__ void credit_task(unsigned long long* tnew, unsigned* 
 // steps, takes its hits from their popcounts over its positions at the end.
 // Each task's hits go once to tnew[i]; per-entry hits to the counters cnt.
 // ---------------------------------------------------------------------------
-template <bool PV, bool WIN, class Tab>
-__device__ __forceinline__ void warp_probe_group(const Task* __restrict__ tasks, int64_t tb, int64_t t1,
+template <bool PV, bool WIN, bool WHOLE, class Tab>
+__device__ __forceinline__ void warp_probe_group(const GraphView& G, const Task* __restrict__ tasks, int64_t tb, int64_t t1,
                                                  const int32_t* __restrict__ adj, const Tab& T,
                                                  unsigned* cnt, unsigned long long* tnew, unsigned* tlow,
                                                  int64_t* s_base, int64_t t0, unsigned short* defer,
@@ -459,7 +471,7 @@ __device__ __forceinline__ void warp_probe_group(const Task* __restrict__ tasks,
     if (valid) {
         const Task tk = tasks[t];
         start = tk.start;
-        len = tk.len;
+        len = tail_length<WHOLE>(G, tk);
         i = tk.i;
         if (WIN) {
             // a tile of a host-resident graph: rows outside its block wait
@@ -549,11 +561,6 @@ __device__ __forceinline__ void warp_probe_group(const Task* __restrict__ tasks,
     if (PV && valid && c) credit_task(tnew, tlow, i, c);
 }
 
-__device__ __forceinline__ int64_t off_at(const GraphView& G, int64_t v) {
-    return G.off64 ? static_cast<const int64_t*>(G.off)[v]
-                   : (int64_t) static_cast<const int32_t*>(G.off)[v];
-}
-
 // Per-warp running total of hits bound for one counter (a graph's total, or
 // a component's total), flushed when the warp moves to a unit whose hits go
 // elsewhere (and at the end).  Every triangle found at pivot j lies in j's
@@ -623,7 +630,7 @@ __device__ __forceinline__ void warp_unit(const GraphView& G, const Unit& U, uns
         __syncwarp();
         const BitTab T{region, pre, lo, hi};
         for (int64_t tb = U.t0; tb < U.t1; tb += 32)
-            warp_probe_group<PV, WIN>(G.tasks, tb, U.t1, G.adj, T, cnt, G.tnew, tlow, s_base, U.t0, nullptr,
+            warp_probe_group<PV, WIN, false>(G, G.tasks, tb, U.t1, G.adj, T, cnt, G.tnew, tlow, s_base, U.t0, nullptr,
                                       nullptr, uh, probes, TaskWindow{G.i0, G.i1, G.tail_shift});
         __syncwarp();
         if (PV) {
@@ -646,7 +653,7 @@ __device__ __forceinline__ void warp_unit(const GraphView& G, const Unit& U, uns
         __syncwarp();
         const HashTab T{tab, bmask, lo, hi};
         for (int64_t tb = U.t0; tb < U.t1; tb += 32)
-            warp_probe_group<PV, WIN>(G.tasks, tb, U.t1, G.adj, T, cnt, G.tnew, tlow, s_base, U.t0, nullptr,
+            warp_probe_group<PV, WIN, false>(G, G.tasks, tb, U.t1, G.adj, T, cnt, G.tnew, tlow, s_base, U.t0, nullptr,
                                       nullptr, uh, probes, TaskWindow{G.i0, G.i1, G.tail_shift});
         __syncwarp();
         if (PV)
@@ -671,7 +678,7 @@ __device__ __forceinline__ void warp_unit(const GraphView& G, const Unit& U, uns
 // time, with later tasks' records already loading and the next tail
 // prefetched into L2 while the current tail is walked.
 // ---------------------------------------------------------------------------
-template <bool PV, bool WIN, class Tab>
+template <bool PV, bool WIN, bool WHOLE, class Tab>
 __device__ __forceinline__ void cta_probe_unit(const GraphView& G, const Unit& U, const Tab& T,
                                                unsigned* cnt, int* s_ctl, int64_t* s_base,
                                                unsigned short* s_long, unsigned* tlow, uint64_t& uh,
@@ -686,7 +693,7 @@ __device__ __forceinline__ void cta_probe_unit(const GraphView& G, const Unit& U
         g = __shfl_sync(0xffffffffu, g, 0);
         const int64_t tb = U.t0 + (int64_t)g * 32;
         if (tb >= U.t1) break;
-        warp_probe_group<PV, WIN>(tasks, tb, U.t1, adj, T, cnt, G.tnew, tlow, s_base, U.t0, s_long,
+        warp_probe_group<PV, WIN, WHOLE>(G, tasks, tb, U.t1, adj, T, cnt, G.tnew, tlow, s_base, U.t0, s_long,
                                   &s_ctl[1], uh, probes, TaskWindow{G.i0, G.i1, G.tail_shift});
     }
     __syncthreads();
@@ -703,6 +710,7 @@ __device__ __forceinline__ void cta_probe_unit(const GraphView& G, const Unit& U
         t.len = 0;
         if (x < nlong) {
             t = tasks[U.t0 + s_long[x]];
+            t.len = tail_length<WHOLE>(G, t);
             t.start -= shift;
         }
         return t;
@@ -735,6 +743,7 @@ __device__ __forceinline__ void cta_probe_unit(const GraphView& G, const Unit& U
         cur.len = 0;
         if (x < nlong) {
             cur = tasks[U.t0 + s_long[x]];
+            cur.len = tail_length<WHOLE>(G, cur);
             cur.start -= shift;
         }
         while (x < nlong) {
@@ -743,6 +752,7 @@ __device__ __forceinline__ void cta_probe_unit(const GraphView& G, const Unit& U
             nxt.len = 0;
             if (xn < nlong) {
                 nxt = tasks[U.t0 + s_long[xn]];
+                nxt.len = tail_length<WHOLE>(G, nxt);
                 nxt.start -= shift;
                 if (32 * lane < nxt.len)
                     asm volatile("prefetch.global.L2 [%0];" ::"l"(adj + nxt.start + 32 * lane));
@@ -807,7 +817,7 @@ __device__ __forceinline__ void cta_unit(const GraphView& G, const Unit& U, int 
             __syncthreads();
         }
         const BitTab T{region, pre, lo, hi};
-        cta_probe_unit<PV, WIN>(G, U, T, cnt, s_ctl, s_base, s_long, tlow, uh, probes);
+        cta_probe_unit<PV, WIN, false>(G, U, T, cnt, s_ctl, s_base, s_long, tlow, uh, probes);
         __syncthreads();
         if (PV)
             for (int r = threadIdx.x; r < dp; r += blockDim.x) {
@@ -862,7 +872,7 @@ __device__ __forceinline__ void cta_unit(const GraphView& G, const Unit& U, int 
             }
             __syncthreads();
             const TagTab T{region, t2, G.adj + sr, sd, s1, m1};
-            cta_probe_unit<PV, WIN>(G, U, T, cnt, s_ctl, s_base, s_long, tlow, uh, probes);
+            cta_probe_unit<PV, WIN, false>(G, U, T, cnt, s_ctl, s_base, s_long, tlow, uh, probes);
             __syncthreads();
             if (PV)
                 for (int r = threadIdx.x; r < sd; r += blockDim.x) {
@@ -879,7 +889,7 @@ __device__ __forceinline__ void cta_unit(const GraphView& G, const Unit& U, int 
         for (int q = threadIdx.x; q < dp; q += blockDim.x) hash_insert(tab, bmask, G.adj[rb + q]);
         __syncthreads();
         const HashTab T{tab, bmask, lo, hi};
-        cta_probe_unit<PV, WIN>(G, U, T, cnt, s_ctl, s_base, s_long, tlow, uh, probes);
+        cta_probe_unit<PV, WIN, BUCKETS && !WIN>(G, U, T, cnt, s_ctl, s_base, s_long, tlow, uh, probes);
         __syncthreads();
         if (PV)
             for (int s = threadIdx.x; s < 4 * (int)buckets; s += blockDim.x) {
@@ -1034,7 +1044,7 @@ __device__ __forceinline__ void mid_probe(const GraphView& G, const Unit& U, con
     const int lane = threadIdx.x & 31;
     uint64_t uh = 0;
     for (int64_t tb = U.t0; tb < U.t1; tb += 32)
-        warp_probe_group<PV, false>(G.tasks, tb, U.t1, G.adj, T, cnt, G.tnew, tlow, s_base, U.t0, nullptr, nullptr,
+        warp_probe_group<PV, false, false>(G, G.tasks, tb, U.t1, G.adj, T, cnt, G.tnew, tlow, s_base, U.t0, nullptr, nullptr,
                                     uh, probes, TaskWindow{0, 0, 0});
     hits += uh;
     __syncwarp();
@@ -1382,7 +1392,7 @@ __global__ void k_unit_counts(const GraphView* __restrict__ views, const int64_t
         const GraphView& G = views[g];
         const int64_t j = v - vpre[g];
         int64_t a, b, c;
-        unit_split(rule, G.zrow != nullptr, off_at(G, j + 1) - off_at(G, j), G.loff[j + 1] - G.loff[j], a, b, c);
+        unit_split(rule, rule.zones && G.zrow != nullptr, off_at(G, j + 1) - off_at(G, j), G.loff[j + 1] - G.loff[j], a, b, c);
         cs[x] = (int32_t)a;
         cl[x] = (int32_t)b;
         cz[x] = (int32_t)c;
@@ -1403,7 +1413,7 @@ __global__ void k_unit_fill(const GraphView* __restrict__ views, const int64_t* 
         const int64_t dp = off_at(G, j + 1) - off_at(G, j);
         const int64_t a = G.loff[j], b = G.loff[j + 1];
         int64_t ns, nl, nw;
-        unit_split(rule, G.zrow != nullptr, dp, b - a, ns, nl, nw);
+        unit_split(rule, rule.zones && G.zrow != nullptr, dp, b - a, ns, nl, nw);
         if (nw > 0) {
             int64_t p = pz[x];
             for (int64_t t = a; t < b; t += rule.wide_tasks)
@@ -1433,6 +1443,7 @@ UnitRule unit_rule(const tc_tuning& t, bool win, bool zones) {
     r.cta_tasks = t.cta_unit_tasks;
     r.wide_tasks = kZoneTasks;
     r.slice = t.slice_max;
+    r.zones = t.table_mode == 1 ? 0 : 1;
     return r;
 }
 
@@ -1634,6 +1645,7 @@ void count_components(tc_graph* g, const tc_tuning& t, uint64_t* comp_totals_dev
     const UnitLists L = units_of(g);
     launch_count(g->view_comp, L, tt, false, g->counters, st, true, nullptr);
     launch_zone(g->view_comp, L, false, g->counters, st, nullptr, true);
+    g->zone_probes = L.nzone > 0 ? g->covered : 0;
     TC_CUDA(cudaMemcpyAsync(comp_totals_dev, g->comp_totals, sizeof(uint64_t) * (size_t)g->num_comps,
                             cudaMemcpyDeviceToDevice, st));
 }
@@ -1659,6 +1671,7 @@ void count(tc_graph* g, const tc_tuning& t, uint64_t* total_dev, uint64_t* per_v
     const UnitLists L = units_of(g);
     launch_count(g->view, L, tt, pv, g->counters, st, true, tlow32 ? g->tlow : nullptr);
     launch_zone(g->view, L, pv, g->counters, st, tlow32 ? g->tlow : nullptr, true);
+    g->zone_probes = L.nzone > 0 ? g->covered : 0;
     if (pv && g->n > 0) {
         {
             Prof prof_("k_gather_pv", st);

@@ -130,6 +130,7 @@ static_assert(kFlatWork / 64 >= 16, "a wide pivot of few entries has at least 16
 struct UnitRule {
     int small_max, mid_max;   // mid_max 0: no wide pivots but the zones' own
     int warp_tasks, cta_tasks, wide_tasks, slice;
+    int zones;                // 0: a graph's zones are not used (its lists are read whole)
 };
 
 __host__ __device__ __forceinline__ void unit_split(const UnitRule& r, bool zoned, int64_t dp, int64_t nt,

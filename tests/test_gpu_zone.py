@@ -102,3 +102,36 @@ def test_dense_graph_beyond_the_persistent_form(tc, k):
     total, t = g.count(per_vertex=True)
     assert total == k * (k - 1) * (k - 2) // 6 and bool((t == (k - 1) * (k - 2) // 2).all())
     g.free()
+
+
+def launched(tc, call):
+    tc.profile_enable()
+    out = call()
+    torch.cuda.synchronize()
+    names = set(tc.profile_read())
+    tc.profile_enable(False)
+    return out, names
+
+
+@pytest.mark.parametrize("small_max", [1, 16, 64])
+def test_hashed_pivots_use_no_zones(tc, small_max):
+    """table_mode 1 is the AND-hash alone, in a graph that has zones too; the
+    work counters are those of the last count."""
+    hs, hd, n = hub_graph(3000, 6000, 90, 0.2, 8)
+    want, want_t = oracle.count(hs, hd, n, per_vertex=True)
+    g = tc.preprocess(torch.from_numpy(hs).cuda(), torch.from_numpy(hd).cuda(), n)
+    t = tc.tuning_default()
+    t.table_mode, t.small_max_outdeg = 1, small_max
+    (total, pv), names = launched(tc, lambda: g.count(per_vertex=True, tuning=t))
+    assert total == want and np.array_equal(pv.cpu().numpy().astype(np.uint64), want_t)
+    assert not names & {"k_zone", "k_light"}, names
+    hashed = sum(g.count_stats()["probes"])
+    b = tc.Batch([g, g], tuning=t)
+    assert b.count().tolist() == [want, want]
+    assert sum(b.count_stats()["probes"]) == 2 * hashed
+    b.free()
+    total, names = launched(tc, g.count)
+    assert total == want and {"k_zone", "k_light"} <= names
+    assert sum(g.count_stats()["probes"]) == hashed
+    assert g.count(tuning=t) == want and sum(g.count_stats()["probes"]) == hashed
+    g.free()
