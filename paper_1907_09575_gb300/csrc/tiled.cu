@@ -114,12 +114,12 @@ void graph_offload(tc_graph* g, cudaStream_t st) {
     const int64_t n = g->n, m = g->m, T = g->n_tasks;
     const size_t ob = g->off64 ? 8 : 4;
     try {
-        zone_restore(g, st);
         take(&h->off, ob * (size_t)(n + 1));
         take(reinterpret_cast<void**>(&h->adj), 4 * (size_t)m);
         take(reinterpret_cast<void**>(&h->loff), 8 * (size_t)(n + 1));
         take(reinterpret_cast<void**>(&h->tasks), sizeof(Task) * (size_t)T);
         take(reinterpret_cast<void**>(&h->perm), 4 * (size_t)n);
+        zone_restore(g, st);   // a graph whose copy got no memory stays as it was
         TC_CUDA(cudaMemcpyAsync(h->off, g->off, ob * (size_t)(n + 1), cudaMemcpyDeviceToHost, st));
         if (m) TC_CUDA(cudaMemcpyAsync(h->adj, g->adj, 4 * (size_t)m, cudaMemcpyDeviceToHost, st));
         TC_CUDA(cudaMemcpyAsync(h->loff, g->loff, 8 * (size_t)(n + 1), cudaMemcpyDeviceToHost, st));
