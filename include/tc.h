@@ -95,8 +95,9 @@ typedef struct {
                                   label); 1: the AND-hash of Section 5.2 in 4-slot
                                   buckets for every pivot (the hashed-pivot
                                   ablation: no bitmaps, no dense zones) */
-    int32_t merge_max_outdeg;  /* accepted (<= 64) and without effect: the rows of
-                                  warp units are searched at any size */
+    int32_t merge_max_outdeg;  /* pivots with |U_j| <= this (<= 64) get no table: a warp
+                                  searches their rows; 0: the tasks of a pivot decide
+                                  (not used with table_mode 1) */
     int32_t reserved;
 } tc_tuning;
 
@@ -372,8 +373,8 @@ TC_API tc_status tc_generate_rmat(uint64_t seed, int32_t scale, int64_t n, int64
  *   receives num device uint64 totals, in the order the graphs were given.
  *   Stream ordered; one count at a time per batch.
  * tc_batch_autotune: times candidate tunings (reps replays each: warp/CTA
- *   bin boundary, tasks per warp and per CTA unit, CTA threads) and keeps the
- *   fastest; the choice is cached per degree profile (graph count, mean
+ *   bin boundary, tasks per warp and per CTA unit, CTA threads, and whether the
+ *   shortest rows may have tables) and keeps the fastest; the choice is cached per degree profile (graph count, mean
  *   edges, largest pivot row, mean tail length) for later batches in the
  *   process.  *chosen (may be NULL) receives it.  Synchronises `stream`.
  * tc_batch_get_count_stats: work counters of the last tc_batch_count;

@@ -701,7 +701,7 @@ __device__ void tasks_sum(const BuildArgs& a) {
         long long nt = 0;
         int64_t x, y, z;
         for (int c = 0; c < a.tcopies; ++c) nt += a.tcur[c * a.n + r];
-        unit_split(a.rule, a.zcap > 0, a.dplus[r], nt, x, y, z);
+        unit_split<false>(a.rule, a.zcap > 0, a.dplus[r], nt, x, y, z);
         t += nt;
         us += x;
         ul += y;
@@ -860,7 +860,7 @@ __device__ void phase_units(const BuildArgs& a) {
             const int64_t dp = row_begin(a, j + 1) - row_begin(a, j);
             b0 = a.loff[j];
             b1 = a.loff[j + 1];
-            unit_split(a.rule, a.zcap > 0, dp, b1 - b0, us, ul, uz);
+            unit_split<false>(a.rule, a.zcap > 0, dp, b1 - b0, us, ul, uz);
             slices = (dp + a.rule.slice - 1) / a.rule.slice;
         }
         const long long xs = cs + block_scan(us, &ts), xl = cl + block_scan(ul, &tl);

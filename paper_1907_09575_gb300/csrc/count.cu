@@ -1392,7 +1392,7 @@ __global__ void k_unit_counts(const GraphView* __restrict__ views, const int64_t
         const GraphView& G = views[g];
         const int64_t j = v - vpre[g];
         int64_t a, b, c;
-        unit_split(rule, rule.zones && G.zrow != nullptr, off_at(G, j + 1) - off_at(G, j), G.loff[j + 1] - G.loff[j], a, b, c);
+        unit_split<true>(rule, rule.zones && G.zrow != nullptr, off_at(G, j + 1) - off_at(G, j), G.loff[j + 1] - G.loff[j], a, b, c);
         cs[x] = (int32_t)a;
         cl[x] = (int32_t)b;
         cz[x] = (int32_t)c;
@@ -1413,7 +1413,7 @@ __global__ void k_unit_fill(const GraphView* __restrict__ views, const int64_t* 
         const int64_t dp = off_at(G, j + 1) - off_at(G, j);
         const int64_t a = G.loff[j], b = G.loff[j + 1];
         int64_t ns, nl, nw;
-        unit_split(rule, rule.zones && G.zrow != nullptr, dp, b - a, ns, nl, nw);
+        unit_split<true>(rule, rule.zones && G.zrow != nullptr, dp, b - a, ns, nl, nw);
         if (nw > 0) {
             int64_t p = pz[x];
             for (int64_t t = a; t < b; t += rule.wide_tasks)
@@ -1438,6 +1438,7 @@ __global__ void k_unit_fill(const GraphView* __restrict__ views, const int64_t* 
 UnitRule unit_rule(const tc_tuning& t, bool win, bool zones) {
     UnitRule r;
     r.small_max = t.small_max_outdeg;
+    r.merge_max = t.merge_max_outdeg;
     r.mid_max = win || t.table_mode == 1 || !zones ? 0 : kMidMaxOutdeg;
     r.warp_tasks = t.warp_unit_tasks;
     r.cta_tasks = t.cta_unit_tasks;
@@ -1576,8 +1577,9 @@ CountLaunch prepare_count(const UnitLists& L, const tc_tuning& t, bool pv, bool 
     c.pv = pv;
     c.buckets = t.table_mode == 1;
     c.win = win;
-    // a graph with CTA units but no wide ones is small: one kernel for all
-    c.light = !c.win && !c.buckets && (L.nzone > 0 || L.nlarge == 0);
+    // a graph with CTA units but no wide ones is small: one kernel for all,
+    // unless its short rows are to be searched
+    c.light = !c.win && !c.buckets && (L.nzone > 0 || L.nlarge == 0 || t.merge_max_outdeg > 0);
     auto kern = count_kernel(pv, c.win, c.buckets, !c.light);
     TC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.smem));
     int per_sm = 0;

@@ -129,15 +129,19 @@ static_assert(kFlatWork / 64 >= 16, "a wide pivot of few entries has at least 16
 
 struct UnitRule {
     int small_max, mid_max;   // mid_max 0: no wide pivots but the zones' own
+    int merge_max;            // pivots of at most this many entries get no table
     int warp_tasks, cta_tasks, wide_tasks, slice;
     int zones;                // 0: a graph's zones are not used (its lists are read whole)
 };
 
+// MERGE: the rule has a merge_max (the one preprocessing plans for has none).
+template <bool MERGE>
 __host__ __device__ __forceinline__ void unit_split(const UnitRule& r, bool zoned, int64_t dp, int64_t nt,
                                                     int64_t& small, int64_t& large, int64_t& wide) {
     small = large = wide = 0;
     if (dp <= 0 || nt <= 0) return;
-    const bool mid = dp <= r.mid_max && (dp > kZoneMinPivot || (dp <= r.small_max && dp * nt >= kFlatWork));
+    const bool tabled = dp <= r.small_max && (!MERGE || dp > r.merge_max) && dp * nt >= kFlatWork;
+    const bool mid = dp <= r.mid_max && (dp > kZoneMinPivot || tabled);
     if (mid || (zoned && dp > kZoneMinPivot)) wide = (nt + r.wide_tasks - 1) / r.wide_tasks;
     if (mid) return;
     if (dp <= r.small_max) small = (nt + r.warp_tasks - 1) / r.warp_tasks;

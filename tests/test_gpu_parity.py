@@ -358,3 +358,43 @@ def test_pinned_host_input_paths(tc):
         assert tm["input_pinned"] and tm["h2d_ms"] >= 0 and tm["count_ms"] > 0
     total3 = tc.triangles(hs, hd, spec.n)   # pageable
     assert total3 == want and not tc.triangles_timing()["input_pinned"]
+
+
+@pytest.mark.parametrize("pairs", [1 << 17, 1 << 21])
+@pytest.mark.parametrize("merge", [0, 8, 64])
+def test_short_rows_searched(tc, pairs, merge):
+    """merge_max_outdeg: pivots of up to that many entries get no table, in a
+    small graph (whose warp units k_count would table) and in one with zones
+    (whose pivots of few entries and many tasks k_light would)."""
+    hs, hd = inputs.rmat(9, 14, pairs)
+    n = 1 << 14
+    lo, hi = np.minimum(hs, hd).astype(np.int64), np.maximum(hs, hd).astype(np.int64)
+    key = np.unique((lo * n + hi)[lo != hi])
+    lo, hi = key // n, key % n
+    deg = np.bincount(lo, minlength=n) + np.bincount(hi, minlength=n)
+    label = np.empty(n, np.int64)
+    label[np.argsort(deg, kind="stable")] = np.arange(n)
+    key = np.sort(np.minimum(label[lo], label[hi]) * n + np.maximum(label[lo], label[hi]))
+    row, col = key // n, key % n
+    task = np.append(row[1:] == row[:-1], False)      # entries of the row follow
+    tasks, length = np.bincount(col[task], minlength=n), np.bincount(row, minlength=n)
+    count = {k: int(tasks[(length > 0) & (length <= k)].sum()) for k in (merge, 64)}
+    g = tc.preprocess(torch.from_numpy(hs).cuda(), torch.from_numpy(hd).cuda(), n)
+    t = tc.Tuning()
+    t.merge_max_outdeg = merge
+    tc.profile_enable()
+    total, tv = g.count(per_vertex=True, tuning=t)
+    names = set(tc.profile_read())
+    tc.profile_enable(False)
+    want, want_t = oracle.count(hs, hd, n, per_vertex=True)
+    assert total == want and np.array_equal(tv.cpu().numpy().astype(np.uint64), want_t)
+    searched = g.count_stats()["tasks"][0]
+    assert ("k_light" in names) == (merge > 0 or pairs > 1 << 19)
+    if "k_light" in names:
+        assert count[merge] <= searched <= count[64]
+        if merge == 64:
+            assert searched == count[64]
+    b = tc.Batch([g, g], tuning=t)
+    assert b.count().tolist() == [want, want]
+    b.free()
+    g.free()
