@@ -233,6 +233,7 @@ tc_status tc_preprocess(const int32_t* src, const int32_t* dst, int64_t num_pair
     g->stats.num_pairs = num_pairs;
     try {
         preprocess(g, src, dst, num_pairs, flags, static_cast<cudaStream_t>(stream));
+        graph_trim(g, static_cast<cudaStream_t>(stream));
     } catch (...) {
         graph_release(g);
         throw;
@@ -274,6 +275,7 @@ tc_status tc_preprocess_components(const int32_t* src, const int32_t* dst, int64
     try {
         preprocess_with_components(g, src, dst, num_pairs, flags, vertex_prefix, num_comps,
                                    static_cast<cudaStream_t>(stream));
+        graph_trim(g, static_cast<cudaStream_t>(stream));
     } catch (...) {
         graph_release(g);
         throw;

@@ -1043,7 +1043,7 @@ void build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64_t P,
     }
     g->plan_m = cap_m;
     const tc_tuning tt = clamp_tuning(size_tuning(def, cap_m));
-    graph_arena(g, cap_m, off64, num_comps);
+    graph_arena(g, cap_m, zone_capacity(cap_m), off64, num_comps);
     a.off = g->off;
     a.adj = g->adj;
     a.perm = g->perm;
@@ -1088,6 +1088,7 @@ void build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64_t P,
     g->n_large = h.nlarge;
     g->n_zone = h.nzone;
     g->covered = h.covered;
+    g->zone_blocks = h.nblocks;
     g->m = (int64_t)h.m;
     g->n_tasks = (int64_t)h.tasks;
     g->stats.m = g->m;

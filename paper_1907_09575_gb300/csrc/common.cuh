@@ -173,7 +173,8 @@ struct tc_graph {
     unsigned* tlow = nullptr;   // 32-bit per-task shares (per-vertex counts), n, on demand
     size_t tlow_bytes = 0;
     // dense zones (zone.cuh); zcap = 0: none
-    int64_t zcap = 0;           // blocks there is room for
+    int64_t zcap = 0;           // blocks there is room for ...
+    int64_t zone_blocks = 0;    // ... and were wanted (zcap, where that is sized by the edges)
     uint2* zrow = nullptr;      // per row: blocks, first zoned edge
     uint32_t* zbits = nullptr;
     uint32_t* zowner = nullptr; // row of a row's first block

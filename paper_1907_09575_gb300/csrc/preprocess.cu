@@ -20,6 +20,7 @@
 #include <algorithm>
 #include <chrono>
 #include <cstring>
+#include <utility>
 
 #include "common.cuh"
 #include "tc_internal.cuh"
@@ -753,54 +754,95 @@ __global__ void k_comp_new(const int32_t* __restrict__ perm, int64_t n, const in
         comp[perm[v]] = comp_of(vpre, num, v);
 }
 
+// The arrays of a graph to another arena, 16 bytes at a time: an arena's parts
+// begin and end on 256 bytes, units have 32.  One launch: a copy each took twice
+// as long as the rest (14 of them: 45 us for 2 MB).
+constexpr int kMaxMoves = 12;
+struct Moves {
+    uint4* dst[kMaxMoves];
+    const uint4* src[kMaxMoves];
+    int64_t words[kMaxMoves];
+    int num;
+    GraphView view, view_comp;
+    GraphView *view_at, *view_comp_at;
+};
+
+__global__ void __launch_bounds__(kT) k_move(const __grid_constant__ Moves mv) {
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, T = (int64_t)gridDim.x * blockDim.x;
+    for (int a = 0; a < mv.num; ++a)
+        for (int64_t q = t; q < mv.words[a]; q += T) mv.dst[a][q] = mv.src[a][q];
+    if (t == 0) {
+        *mv.view_at = mv.view;
+        *mv.view_comp_at = mv.view_comp;
+    }
+}
+
 }  // namespace
 
-void graph_arena(tc_graph* g, int64_t cap_m, bool off64, int32_t num_comps) {
-    const size_t n = (size_t)g->n, nv = std::max<size_t>(n, 1), m = (size_t)std::max<int64_t>(cap_m, 1);
-    const bool low = g->n <= kBuildMaxPairs;   // larger graphs take tlow when they need it
-    size_t need = 0;
-    auto take = [&](size_t bytes) {
-        const size_t at = need;
-        need += align_up(bytes);
+// The arena's parts for up to cap_m edges and zcap zone blocks, in bytes from
+// its start.
+struct ArenaPlan {
+    size_t off, adj, perm, loff, tasks, view, view_comp, zrow, zbits, zowner, comp, counters, comp_totals, tnew, tlow;
+    size_t bytes = 0;
+    bool low;   // tlow inside; larger graphs take it when they need it
+
+    ArenaPlan(int64_t n, int64_t cap_m, int64_t zcap, bool off64, int32_t num_comps) {
+        const size_t nv = (size_t)std::max<int64_t>(n, 1), m = (size_t)std::max<int64_t>(cap_m, 1);
+        low = n <= kBuildMaxPairs;
+        off = take((off64 ? 8 : 4) * (size_t)(n + 1));
+        adj = take(4 * m);
+        perm = take(4 * nv);
+        loff = take(8 * (size_t)(n + 1));
+        tasks = take(sizeof(Task) * m);
+        view = take(sizeof(GraphView));
+        view_comp = take(sizeof(GraphView));
+        zrow = take(zcap ? 8 * nv : 0);
+        zbits = take(4 * (size_t)kZoneWords * (size_t)zcap);
+        zowner = take(4 * (size_t)zcap);
+        comp = take(num_comps > 0 ? 4 * nv : 0);
+        counters = take(sizeof(unsigned long long) * CTR_COUNT);
+        comp_totals = take(8 * (size_t)std::max(num_comps, 0));
+        tnew = take(8 * nv);
+        tlow = take(low ? 4 * nv : 0);
+    }
+
+private:
+    size_t take(size_t size) {
+        const size_t at = bytes;
+        bytes += align_up(size);
         return at;
-    };
-    const size_t o_off = take((off64 ? 8 : 4) * (n + 1)), o_adj = take(4 * m), o_perm = take(4 * nv);
-    const size_t o_loff = take(8 * (n + 1)), o_tasks = take(sizeof(Task) * m);
-    const size_t o_view = take(sizeof(GraphView)), o_vc = take(sizeof(GraphView));
-    const int64_t zcap = zone_capacity(cap_m);
-    const size_t o_zrow = take(zcap ? 8 * nv : 0);
-    const size_t o_zbits = take(4 * (size_t)kZoneWords * (size_t)zcap), o_zown = take(4 * (size_t)zcap);
-    const size_t o_comp = take(num_comps > 0 ? 4 * nv : 0);
-    const size_t o_ctr = take(sizeof(unsigned long long) * CTR_COUNT);
-    const size_t o_ctot = take(8 * (size_t)std::max(num_comps, 0));
-    const size_t o_tnew = take(8 * nv), o_tlow = take(low ? 4 * nv : 0);
+    }
+};
+
+void graph_arena(tc_graph* g, int64_t cap_m, int64_t zcap, bool off64, int32_t num_comps) {
+    const ArenaPlan p(g->n, cap_m, zcap, off64, num_comps);
+    char* a = static_cast<char*>(g->alloc.get(p.bytes));
+    g->arena = a;
+    g->arena_bytes = p.bytes;
     g->off64 = off64;
-    g->arena_bytes = need;
-    g->arena = g->alloc.get(need);
-    char* a = static_cast<char*>(g->arena);
-    g->off = a + o_off;
-    g->adj = reinterpret_cast<int32_t*>(a + o_adj);
-    g->perm = reinterpret_cast<int32_t*>(a + o_perm);
-    g->loff = reinterpret_cast<int64_t*>(a + o_loff);
-    g->tasks = reinterpret_cast<Task*>(a + o_tasks);
-    g->view = reinterpret_cast<GraphView*>(a + o_view);
-    g->view_comp = reinterpret_cast<GraphView*>(a + o_vc);
-    g->counters = reinterpret_cast<unsigned long long*>(a + o_ctr);
-    g->tnew = reinterpret_cast<uint64_t*>(a + o_tnew);
-    g->zero_bytes = need - o_ctr;
+    g->off = a + p.off;
+    g->adj = reinterpret_cast<int32_t*>(a + p.adj);
+    g->perm = reinterpret_cast<int32_t*>(a + p.perm);
+    g->loff = reinterpret_cast<int64_t*>(a + p.loff);
+    g->tasks = reinterpret_cast<Task*>(a + p.tasks);
+    g->view = reinterpret_cast<GraphView*>(a + p.view);
+    g->view_comp = reinterpret_cast<GraphView*>(a + p.view_comp);
+    g->counters = reinterpret_cast<unsigned long long*>(a + p.counters);
+    g->tnew = reinterpret_cast<uint64_t*>(a + p.tnew);
+    g->zero_bytes = p.bytes - p.counters;
     g->zcap = zcap;
     if (zcap > 0) {
-        g->zrow = reinterpret_cast<uint2*>(a + o_zrow);
-        g->zbits = reinterpret_cast<uint32_t*>(a + o_zbits);
-        g->zowner = reinterpret_cast<uint32_t*>(a + o_zown);
+        g->zrow = reinterpret_cast<uint2*>(a + p.zrow);
+        g->zbits = reinterpret_cast<uint32_t*>(a + p.zbits);
+        g->zowner = reinterpret_cast<uint32_t*>(a + p.zowner);
     }
-    if (low) {
-        g->tlow = reinterpret_cast<unsigned*>(a + o_tlow);
+    if (p.low) {
+        g->tlow = reinterpret_cast<unsigned*>(a + p.tlow);
         g->tlow_in_arena = true;
     }
     if (num_comps > 0) {
-        g->comp = reinterpret_cast<int32_t*>(a + o_comp);
-        g->comp_totals = reinterpret_cast<unsigned long long*>(a + o_ctot);
+        g->comp = reinterpret_cast<int32_t*>(a + p.comp);
+        g->comp_totals = reinterpret_cast<unsigned long long*>(a + p.comp_totals);
         g->num_comps = num_comps;
     }
 }
@@ -822,6 +864,69 @@ void graph_views(const tc_graph* g, GraphView* v, GraphView* vc) {
     vc->tnew = nullptr;
     vc->comp = g->comp;
     vc->comp_totals = g->comp_totals;
+}
+
+// Preprocessing in one launch sizes the arena by the pairs and the units by
+// their bound.  A graph that is kept moves to what its edges need when it holds
+// over half as much again, and 8 MiB: pairs given many times, or few pairs a
+// vertex (RMAT scale 14, 65,536 pairs 64 times: 93.1 MB -> 2.0; scale 20 of
+// 2^20 pairs: 97.4 -> 61.2).
+void graph_trim(tc_graph* g, cudaStream_t st) {
+    if (!g->arena || !g->units_mem) return;
+    const int64_t units = std::max<int64_t>(g->n_large + g->n_zone + g->n_small, 1);
+    const int64_t zcap = g->zcap > 0 ? std::min(g->zcap, g->zone_blocks + 1) : 0;
+    const size_t held = g->arena_bytes + g->units_bytes;
+    const size_t need = ArenaPlan(g->n, g->m, zcap, g->off64, g->num_comps).bytes + sizeof(Unit) * (size_t)units;
+    if (held < need + std::max<size_t>(need / 2, 8 << 20)) return;
+    const tc_graph old = *g;
+    UnitLists L = units_of(g);
+    L.mem = nullptr;
+    L.bytes = sizeof(Unit) * (size_t)units;
+    try {
+        L.mem = g->alloc.get(L.bytes);
+        graph_arena(g, g->m, zcap, g->off64, g->num_comps);
+    } catch (const Error& e) {
+        if (L.mem) g->alloc.put(L.mem, L.bytes);
+        if (e.status != TC_ENOMEM) throw;
+        clear_error();   // no room for both: it stays as it is
+        return;
+    }
+    Moves mv{};
+    auto move = [&](void* dst, const void* src, size_t bytes) {
+        mv.dst[mv.num] = static_cast<uint4*>(dst);
+        mv.src[mv.num] = static_cast<const uint4*>(src);
+        mv.words[mv.num++] = (int64_t)((bytes + 15) / 16);
+    };
+    const size_t n = (size_t)g->n, m = (size_t)g->m;
+    move(g->off, old.off, (g->off64 ? 8 : 4) * (n + 1));
+    move(g->adj, old.adj, 4 * m);
+    move(g->perm, old.perm, 4 * n);
+    move(g->loff, old.loff, 8 * (n + 1));
+    move(g->tasks, old.tasks, sizeof(Task) * (size_t)g->n_tasks);
+    if (zcap > 0) {
+        move(g->zrow, old.zrow, sizeof(uint2) * n);
+        move(g->zbits, old.zbits, 4 * (size_t)kZoneWords * (size_t)zcap);
+        move(g->zowner, old.zowner, 4 * (size_t)zcap);
+    }
+    if (g->num_comps > 0) move(g->comp, old.comp, 4 * n);
+    Unit* to = static_cast<Unit*>(L.mem);
+    for (auto part : {std::make_pair(&L.large, L.nlarge), {&L.zone, L.nzone}, {&L.small, L.nsmall}}) {
+        move(to, *part.first, sizeof(Unit) * (size_t)part.second);
+        *part.first = to;
+        to += part.second;
+    }
+    graph_views(g, &mv.view, &mv.view_comp);
+    mv.view_at = g->view;
+    mv.view_comp_at = g->view_comp;
+    {
+        Prof prof_("k_move", st);
+        k_move<<<grid_for((int64_t)(need / 16), kT, (int64_t)num_sms() * 8), kT, 0, st>>>(mv);
+    }
+    const cudaError_t launched = cudaGetLastError();
+    g->alloc.put(old.arena, old.arena_bytes);
+    adopt_units(g, L, g->units_tuning);
+    TC_CUDA(launched);
+    g->stats.device_bytes = (int64_t)(g->arena_bytes + g->units_bytes);
 }
 
 void preprocess(tc_graph* g, const int32_t* src_in, const int32_t* dst_in, int64_t P,
@@ -1021,7 +1126,7 @@ void preprocess_with_components(tc_graph* g, const int32_t* src_in, const int32_
                                                                          : (m >= (int64_t)0x7fffffff);
     const size_t ob = g->off64 ? 8 : 4;
 
-    graph_arena(g, m, g->off64, num_comps);
+    graph_arena(g, m, zone_capacity(m), g->off64, num_comps);
 
     // a4 relabel
     if (n > 0) {
@@ -1264,6 +1369,7 @@ void preprocess_with_components(tc_graph* g, const int32_t* src_in, const int32_
     g->stats.probes_ijk = hprobes[1];
     g->stats.offset_bytes = (int32_t)ob;
     g->covered = hprobes[2];
+    g->zone_blocks = g->zcap;
     UnitLists L = fill_units(plan, ns, nl, nz, al, st);
     adopt_units(g, L, def);
     g->stats.device_bytes = (int64_t)(g->arena_bytes + g->units_bytes);

@@ -38,7 +38,9 @@ void preprocess_with_components(tc_graph* g, const int32_t* src, const int32_t* 
                                 cudaStream_t st);
 // The graph's device arena for up to cap_m edges (offsets, columns, labels,
 // tasks, counters, accumulators, components), and its views into it.
-void graph_arena(tc_graph* g, int64_t cap_m, bool off64, int32_t num_comps);
+void graph_arena(tc_graph* g, int64_t cap_m, int64_t zcap, bool off64, int32_t num_comps);
+// Gives back what a kept graph holds beyond its edges' need (stream-ordered).
+void graph_trim(tc_graph* g, cudaStream_t st);
 void graph_views(const tc_graph* g, GraphView* v, GraphView* vc);
 
 // Preprocessing of graphs of up to kBuildMaxPairs pairs in one persistent

@@ -105,3 +105,77 @@ def test_injected_allocation_failures_leak_nothing(tc):
     g = tc.preprocess(s, d, spec.n)
     assert g.count() == want_total
     g.free()
+
+
+def repeated_pairs(tc, kind):
+    """(src, dst, n) given many times over, and the distinct pairs alone."""
+    if kind == "one":
+        s, d = (torch.full((1,), v, dtype=torch.int32, device="cuda") for v in (3, 5))
+        return (s.repeat(1 << 22), d.repeat(1 << 22), 10), (s, d, 10)
+    scale, pairs, times = {"small": (14, 1 << 16, 16), "zones": (16, 3 << 18, 5)}[kind]
+    s, d = tc.generate_rmat(6, scale, pairs)
+    return (s.repeat(times), d.repeat(times), 1 << scale), (s, d, 1 << scale)
+
+
+@pytest.mark.parametrize("kind", ["one", "small", "zones"])
+@pytest.mark.parametrize("offsets", [None, 64])
+def test_kept_graph_holds_what_its_edges_need(tc, kind, offsets):
+    """A graph that stays holds at most half as much again as its edges need
+    (and 8 MiB), however often its pairs were given, and counts the same."""
+    (s, d, n), (s1, d1, _) = repeated_pairs(tc, kind)
+    once = tc.preprocess(s1, d1, n, offsets=offsets)
+    want, want_t = once.count(per_vertex=True)
+    used = tc.memory_stats(torch.cuda.current_device())["used"]
+    g = tc.preprocess(s, d, n, offsets=offsets)
+    torch.cuda.synchronize()
+    held = tc.memory_stats(torch.cuda.current_device())["used"] - used
+    assert held <= 1.5 * once.stats()["device_bytes"] + (9 << 20), (held, once.stats())
+    assert g.stats()["device_bytes"] <= held
+    assert g.stats()["m"] == once.stats()["m"]
+    total, t = g.count(per_vertex=True)
+    assert total == want and torch.equal(t, want_t)
+    u = tc.tuning_default()
+    u.warp_unit_tasks = 7
+    assert g.count(tuning=u) == want
+    b = tc.Batch([g, once])
+    assert b.count().tolist() == [want, want]
+    b.free()
+    g.offload()
+    assert g.count_tiled(1 << 28)[0] == want
+    g.free()
+    once.free()
+    g = tc.preprocess_components(torch.cat([s, s1 + n]), torch.cat([d, d1 + n]), [0, n, 2 * n], offsets=offsets)
+    assert tc.count_components(g).tolist() == [want, want]
+    g.free()
+
+
+def test_failures_while_a_kept_graph_moves(tc):
+    """As above for a graph that moves to a smaller arena: where that finds no
+    memory the graph stays where it is and counts the same."""
+    (s, d, n), (s1, d1, _) = repeated_pairs(tc, "zones")
+    g = tc.preprocess(s1, d1, n)
+    want, want_t = g.count(per_vertex=True)
+    g.free()
+    kept = []
+    fail_at, completed = 1, False
+    while not completed:
+        fa = FailingAllocator(tc, fail_at)
+        g = None
+        try:
+            g = tc.preprocess(s, d, n, allocator=fa.struct)
+            failed = fa.calls >= fail_at
+            total, t = g.count(per_vertex=True)
+            assert total == want and torch.equal(t, want_t)
+            if failed:
+                kept.append(fail_at)
+            completed = fa.calls < fail_at
+        except tc.TCError as e:
+            assert e.status == tc.TC_ENOMEM, e
+        finally:
+            if g is not None:
+                g.free()
+        torch.cuda.synchronize()
+        assert not fa.live, (fail_at, len(fa.live))
+        fail_at += 1
+        assert fail_at < 500
+    assert len(kept) == 2                  # the units' and the arena's
