@@ -374,9 +374,10 @@ TC_API tc_status tc_generate_rmat(uint64_t seed, int32_t scale, int64_t n, int64
  *   Stream ordered; one count at a time per batch.
  * tc_batch_autotune: times candidate tunings (reps replays each: warp/CTA
  *   bin boundary, tasks per warp and per CTA unit, CTA threads, and whether the
- *   shortest rows may have tables) and keeps the fastest; the choice is cached per degree profile (graph count, mean
- *   edges, largest pivot row, mean tail length) for later batches in the
- *   process.  *chosen (may be NULL) receives it.  Synchronises `stream`.
+ *   shortest rows may have tables) and keeps the fastest; the choice is cached
+ *   per degree profile (graph count, mean edges, largest pivot row, mean tail
+ *   length) for later batches in the process.  *chosen (may be NULL) receives
+ *   it.  Synchronises `stream`.
  * tc_batch_get_count_stats: work counters of the last tc_batch_count;
  *   triangles = sum of the totals.  Synchronises `stream`.
  * tc_count_batch: create, count into totals_dev (required), free.
@@ -397,10 +398,12 @@ TC_API tc_status tc_count_batch(const tc_graph* const* graphs, int32_t num, cons
  * them in ticks: worker threads (one CUDA stream each) take requests from
  * the head of the queue while the tick stays within max_batch requests and
  * max_tick_pairs pairs and the device bytes of all ticks in flight stay
- * within hbm_budget_bytes (each request's footprint is estimated as
- * 64 B per pair + 48 B per vertex); a tick's requests are preprocessed as one
- * disjoint union and counted per component (tc_preprocess_components /
- * tc_count_components).  Ticks on different workers overlap on the device.
+ * within hbm_budget_bytes (each request's footprint is taken as 64 B per pair
+ * + 48 B per vertex; a tick of fewer than about five pairs a vertex takes up to
+ * 50 B per pair + 128 B per vertex where the budget has room for it, and a
+ * slower form within its requests' footprints where not); a tick's requests are
+ * preprocessed as one disjoint union and counted per component
+ * (tc_preprocess_components / tc_count_components).  Ticks on different workers overlap on the device.
  * Results carry the caller-given arrival time and the server-clock times of
  * admission and completion (tc_server_now: seconds since creation).
  *

@@ -954,7 +954,7 @@ void build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64_t P,
                  const int64_t* vpre_host, int32_t num_comps, cudaStream_t st) {
     Alloc& al = g->alloc;
     const int64_t n = g->n;
-    const bool one = P <= kBuildOnePairs;
+    const bool one = P <= kBuildOnePairs && !g->lean;
     tc_tuning def;
     tuning_defaults(&def);
 
@@ -967,7 +967,7 @@ void build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64_t P,
     a.nchunks = (int)std::max<int64_t>(1, (n + a.chunk - 1) / std::max<int64_t>(a.chunk, 1));
     a.cap = 2 * (uint64_t)std::max<int64_t>(P, 512);
     const size_t nv = (size_t)std::max<int64_t>(n, 1);
-    a.tcopies = n <= (1ll << 21) ? kTaskCopies : n <= (1ll << 22) ? 4 : 1;
+    a.tcopies = g->lean ? 1 : n <= (1ll << 21) ? kTaskCopies : n <= (1ll << 22) ? 4 : 1;
     size_t need = 0;
     auto take = [&](size_t bytes) {
         const size_t at = need;
@@ -1043,7 +1043,7 @@ void build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64_t P,
     }
     g->plan_m = cap_m;
     const tc_tuning tt = clamp_tuning(size_tuning(def, cap_m));
-    graph_arena(g, cap_m, zone_capacity(cap_m), off64, num_comps);
+    graph_arena(g, cap_m, g->lean ? 0 : zone_capacity(cap_m), off64, num_comps);
     a.off = g->off;
     a.adj = g->adj;
     a.perm = g->perm;

@@ -202,6 +202,7 @@ struct tc_graph {
     void* units_mem = nullptr;      // small units, then large units
     size_t units_bytes = 0;
     tc_tuning units_tuning{};       // tuning the unit lists were built for
+    bool lean = false;              // preprocess within 64 B a pair and 48 B a vertex, for per-component totals only
     int64_t plan_m = 0;             // edges their size was chosen for (the pairs, where the host knew only those)
     tc_graph_stats stats{};
 };

@@ -1395,7 +1395,7 @@ __global__ void k_unit_counts(const GraphView* __restrict__ views, const int64_t
         unit_split<true>(rule, rule.zones && G.zrow != nullptr, off_at(G, j + 1) - off_at(G, j), G.loff[j + 1] - G.loff[j], a, b, c);
         cs[x] = (int32_t)a;
         cl[x] = (int32_t)b;
-        cz[x] = (int32_t)c;
+        if (cz) cz[x] = (int32_t)c;
     }
 }
 
@@ -1444,7 +1444,7 @@ UnitRule unit_rule(const tc_tuning& t, bool win, bool zones) {
     r.cta_tasks = t.cta_unit_tasks;
     r.wide_tasks = kZoneTasks;
     r.slice = t.slice_max;
-    r.zones = t.table_mode == 1 ? 0 : 1;
+    r.zones = !win && t.table_mode != 1 && zones;
     return r;
 }
 
@@ -1464,10 +1464,10 @@ void plan_units(UnitPlan& P, const GraphView* views_dev, const int64_t* vpre_dev
     P.rule = rule;
     P.cs = Buf<int32_t>(al, (size_t)std::max<int64_t>(V, 1));
     P.cl = Buf<int32_t>(al, (size_t)std::max<int64_t>(V, 1));
-    P.cz = Buf<int32_t>(al, (size_t)std::max<int64_t>(V, 1));
+    if (rule.zones) P.cz = Buf<int32_t>(al, (size_t)std::max<int64_t>(V, 1));
     P.ps = Buf<int64_t>(al, (size_t)(V + 1));
     P.pl = Buf<int64_t>(al, (size_t)(V + 1));
-    P.pz = Buf<int64_t>(al, (size_t)(V + 1));
+    if (rule.zones) P.pz = Buf<int64_t>(al, (size_t)(V + 1));
     if (V > 0) {
         Prof prof_("k_unit_counts", st);
         k_unit_counts<<<grid_for(V, 256, G), 256, 0, st>>>(views_dev, vpre_dev, num, V, rule, P.cs.get(), P.cl.get(),
@@ -1476,7 +1476,7 @@ void plan_units(UnitPlan& P, const GraphView* views_dev, const int64_t* vpre_dev
     TC_LAUNCH_CHECK();
     exclusive_scan2_i32_to_i64(P.cs.get(), P.ps.get(), P.ps.get() + V, P.cl.get(), P.pl.get(), P.pl.get() + V, V,
                                al, st);
-    exclusive_scan_i32_to_i64(P.cz.get(), P.pz.get(), V, P.pz.get() + V, al, st);
+    if (rule.zones) exclusive_scan_i32_to_i64(P.cz.get(), P.pz.get(), V, P.pz.get() + V, al, st);
 }
 
 UnitLists fill_units(UnitPlan& P, int64_t ns, int64_t nl, int64_t nz, Alloc& al, cudaStream_t st) {
@@ -1514,7 +1514,7 @@ UnitLists build_unit_lists(const GraphView* views_dev, const int64_t* vpre_dev, 
     plan_units(P, views_dev, vpre_dev, num, V, rule, al, st);
     int64_t ns = 0, nl = 0, nz = 0;
     TC_CUDA(cudaMemcpyAsync(&ns, P.ps.get() + V, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-    TC_CUDA(cudaMemcpyAsync(&nz, P.pz.get() + V, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+    if (rule.zones) TC_CUDA(cudaMemcpyAsync(&nz, P.pz.get() + V, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     TC_CUDA(cudaMemcpyAsync(&nl, P.pl.get() + V, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     TC_CUDA(cudaStreamSynchronize(st));
     return fill_units(P, ns, nl, nz, al, st);

@@ -786,9 +786,10 @@ struct ArenaPlan {
     size_t bytes = 0;
     bool low;   // tlow inside; larger graphs take it when they need it
 
-    ArenaPlan(int64_t n, int64_t cap_m, int64_t zcap, bool off64, int32_t num_comps) {
+    // totals: no accumulators of per-vertex counts
+    ArenaPlan(int64_t n, int64_t cap_m, int64_t zcap, bool off64, int32_t num_comps, bool totals = false) {
         const size_t nv = (size_t)std::max<int64_t>(n, 1), m = (size_t)std::max<int64_t>(cap_m, 1);
-        low = n <= kBuildMaxPairs;
+        low = !totals && n <= kBuildMaxPairs;
         off = take((off64 ? 8 : 4) * (size_t)(n + 1));
         adj = take(4 * m);
         perm = take(4 * nv);
@@ -802,7 +803,7 @@ struct ArenaPlan {
         comp = take(num_comps > 0 ? 4 * nv : 0);
         counters = take(sizeof(unsigned long long) * CTR_COUNT);
         comp_totals = take(8 * (size_t)std::max(num_comps, 0));
-        tnew = take(8 * nv);
+        tnew = take(totals ? 0 : 8 * nv);
         tlow = take(low ? 4 * nv : 0);
     }
 
@@ -815,7 +816,7 @@ private:
 };
 
 void graph_arena(tc_graph* g, int64_t cap_m, int64_t zcap, bool off64, int32_t num_comps) {
-    const ArenaPlan p(g->n, cap_m, zcap, off64, num_comps);
+    const ArenaPlan p(g->n, cap_m, zcap, off64, num_comps, g->lean);
     char* a = static_cast<char*>(g->alloc.get(p.bytes));
     g->arena = a;
     g->arena_bytes = p.bytes;
@@ -828,7 +829,7 @@ void graph_arena(tc_graph* g, int64_t cap_m, int64_t zcap, bool off64, int32_t n
     g->view = reinterpret_cast<GraphView*>(a + p.view);
     g->view_comp = reinterpret_cast<GraphView*>(a + p.view_comp);
     g->counters = reinterpret_cast<unsigned long long*>(a + p.counters);
-    g->tnew = reinterpret_cast<uint64_t*>(a + p.tnew);
+    g->tnew = g->lean ? nullptr : reinterpret_cast<uint64_t*>(a + p.tnew);
     g->zero_bytes = p.bytes - p.counters;
     g->zcap = zcap;
     if (zcap > 0) {
@@ -1126,7 +1127,7 @@ void preprocess_with_components(tc_graph* g, const int32_t* src_in, const int32_
                                                                          : (m >= (int64_t)0x7fffffff);
     const size_t ob = g->off64 ? 8 : 4;
 
-    graph_arena(g, m, zone_capacity(m), g->off64, num_comps);
+    graph_arena(g, m, g->lean ? 0 : zone_capacity(m), g->off64, num_comps);
 
     // a4 relabel
     if (n > 0) {
@@ -1338,6 +1339,13 @@ void preprocess_with_components(tc_graph* g, const int32_t* src_in, const int32_
         TC_CUDA(cudaMemcpyAsync(g->view_comp, &vc, sizeof(vc), cudaMemcpyHostToDevice, st));
     }
 
+    // what the units need not: their plan is the peak of a graph of few pairs a
+    // vertex
+    off64.release();
+    dplus.release();
+    kb.release();
+    ab.release();
+
     // a6 work units for the default tuning, sized at the same synchronisation
     // as the task statistics
     tc_tuning def;
@@ -1358,7 +1366,8 @@ void preprocess_with_components(tc_graph* g, const int32_t* src_in, const int32_
     TC_CUDA(cudaMemcpyAsync(&ntasks, g->loff + n, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     TC_CUDA(cudaMemcpyAsync(&ns, plan.ps.get() + n, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     TC_CUDA(cudaMemcpyAsync(&nl, plan.pl.get() + n, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-    TC_CUDA(cudaMemcpyAsync(&nz, plan.pz.get() + n, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+    if (plan.rule.zones)
+        TC_CUDA(cudaMemcpyAsync(&nz, plan.pz.get() + n, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     TC_CUDA(cudaStreamSynchronize(st));
     if (herr & 4) TC_FAIL(TC_ETIMEOUT, "tc_preprocess: a sort look-back wait ran past its bound");
     if (herr & 8) TC_FAIL(TC_EUNSUPPORTED, "tc_preprocess: a row of U exceeds the row sort's bound");

@@ -31,11 +31,20 @@ struct Pending {
     int64_t bytes;
 };
 
-int64_t footprint(const tc_rmat_spec& s) {
-    // pairs on the device (8 B), preprocessing scratch (~28 B per pair),
-    // graph arena (~24 B per edge, ~40 B per vertex), plus slack
-    return 64 * s.num_pairs + 48 * s.n + 4096;
-}
+// What a request is admitted by, and what the lean form of preprocessing takes
+// for a tick at most.  Up to 2^24 pairs: the pairs (8 B), the set (16.1 B a
+// pair, 24 B a vertex and 1 B of counts), offsets, columns, labels and tasks (20
+// B an edge, 20 B a vertex), units of 32 B for at most half the edges, and one
+// more for every 16 tasks (18.9 B an edge).  Beyond: 48 B a pair while the set
+// is filled; 44 B a pair and 40 B a vertex after; 28 and 44 with the units' plan
+// and 18.9 more with the units.
+int64_t footprint(const tc_rmat_spec& s) { return 64 * s.num_pairs + 48 * s.n + 4096; }
+
+// What the usual form takes at most, with eight counters of tasks a vertex,
+// zones, accumulators and in one launch the units' bound: 49.1 B a pair and 125
+// B a vertex (beyond 2^24 pairs 49 and 76), above the lean form's below five
+// pairs a vertex.
+int64_t tick_bytes_full(int64_t pairs, int64_t vertices) { return 50 * pairs + 128 * vertices + (64 << 10); }
 
 }  // namespace
 
@@ -68,7 +77,7 @@ namespace {
 
 // Runs one tick on stream st; fills totals (one per request).  e0 and e1 are
 // recorded on st before the tick's first device operation and after its last.
-void run_tick(const std::vector<Pending>& reqs, std::vector<uint64_t>& totals, cudaStream_t st,
+void run_tick(const std::vector<Pending>& reqs, bool lean, std::vector<uint64_t>& totals, cudaStream_t st,
               cudaEvent_t e0, cudaEvent_t e1) {
     const int nreq = (int)reqs.size();
     std::vector<int64_t> ppre(nreq + 1, 0), vpre(nreq + 1, 0);
@@ -93,6 +102,7 @@ void run_tick(const std::vector<Pending>& reqs, std::vector<uint64_t>& totals, c
     tc_graph* g = new tc_graph();
     try {
         g->n = vpre[nreq];
+        g->lean = lean;
         g->num_pairs = P;
         g->bits = std::max(1, ceil_log2_u64((uint64_t)std::max<int64_t>(g->n, 1)));
         g->alloc.stream = st;
@@ -130,6 +140,7 @@ void worker_loop(tc_server* S) {
     while (true) {
         std::vector<Pending> tick;
         int64_t tick_bytes = 0;
+        bool lean = false;
         {
             std::unique_lock<std::mutex> lk(S->mu);
             S->cv.wait(lk, [&] {
@@ -141,7 +152,7 @@ void worker_loop(tc_server* S) {
             if (S->stop && S->pending.empty()) break;
             if (S->stop && S->bytes_in_flight + S->pending.front().bytes > S->cfg.hbm_budget_bytes)
                 break;
-            int64_t pairs = 0;
+            int64_t pairs = 0, vertices = 0;
             while (!S->pending.empty() && (int)tick.size() < S->cfg.max_batch) {
                 const Pending& p = S->pending.front();
                 if (!tick.empty() && pairs + p.spec.num_pairs > S->cfg.max_tick_pairs) break;
@@ -149,8 +160,13 @@ void worker_loop(tc_server* S) {
                 tick.push_back(p);
                 tick_bytes += p.bytes;
                 pairs += p.spec.num_pairs;
+                vertices += p.spec.n;
                 S->pending.pop_front();
             }
+            // requests of few pairs a vertex take the usual form where it fits
+            const int64_t full = std::max(tick_bytes, tick_bytes_full(pairs, vertices));
+            lean = S->bytes_in_flight + full > S->cfg.hbm_budget_bytes;
+            if (!lean) tick_bytes = full;
             S->bytes_in_flight += tick_bytes;
             S->peak_bytes = std::max(S->peak_bytes, S->bytes_in_flight);
             S->busy_workers += 1;
@@ -160,7 +176,7 @@ void worker_loop(tc_server* S) {
         tc_status status = TC_OK;
         double d0 = -1.0, d1 = -1.0;
         try {
-            run_tick(tick, totals, st, e0, e1);
+            run_tick(tick, lean, totals, st, e0, e1);
             float a = 0.f, b = 0.f;
             if (cudaEventElapsedTime(&a, S->ev_ref, e0) == cudaSuccess &&
                 cudaEventElapsedTime(&b, S->ev_ref, e1) == cudaSuccess) {

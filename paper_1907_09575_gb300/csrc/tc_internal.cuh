@@ -70,7 +70,7 @@ struct UnitLists {
 // scans (the list sizes land at ps[V], pl[V], pz[V] on the device); once the host
 // knows them, fill_units allocates and fills the lists.
 struct UnitPlan {
-    Buf<int32_t> cs, cl, cz;
+    Buf<int32_t> cs, cl, cz;   // cz, pz: only by a rule with zones
     Buf<int64_t> ps, pl, pz;
     int64_t V = 0;
     int num = 0;

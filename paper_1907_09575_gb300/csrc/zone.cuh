@@ -131,7 +131,7 @@ struct UnitRule {
     int small_max, mid_max;   // mid_max 0: no wide pivots but the zones' own
     int merge_max;            // pivots of at most this many entries get no table
     int warp_tasks, cta_tasks, wide_tasks, slice;
-    int zones;                // 0: a graph's zones are not used (its lists are read whole)
+    int zones;                // 0: no zones, or not used (lists are read whole), and no wide pivots
 };
 
 // MERGE: the rule has a merge_max (the one preprocessing plans for has none).

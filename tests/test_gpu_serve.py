@@ -179,3 +179,39 @@ def test_admission_and_host_side_failures(tc):
     srv.drain()
     assert srv.stats()["completed"] == 20
     srv.free()
+
+
+def footprint(specs):
+    return sum(64 * m + 48 * n + 4096 for _, _, n, m in specs)
+
+
+@pytest.mark.parametrize("pairs,n", [(1 << 16, 1 << 18), (1 << 20, 1 << 20), (1 << 20, 1 << 19), (3 << 19, 1 << 18),
+                                     ((1 << 22) + 5, 1 << 22), ((1 << 24) + 5, 1 << 24), ((1 << 24) + 5, 1 << 22),
+                                     (1 << 20, (1 << 24) + 9), ((1 << 26) + 5, 1 << 26)])
+@pytest.mark.parametrize("room", [1, 4])
+def test_sparse_requests_stay_within_the_budget(tc, pairs, n, room):
+    """Requests of few pairs a vertex, with a budget that just admits two of
+    them and with a larger one: they are admitted by 64 B per pair and 48 B per
+    vertex, and what the pool hands out stays within the bytes accounted for."""
+    dev = torch.cuda.current_device()
+    specs = [(s, max(1, (n - 1).bit_length()), n, pairs) for s in (1, 2)]
+    budget = footprint(specs) * room
+    torch.cuda.synchronize()
+    tc.memory_stats(dev, reset_high=True)
+    base = tc.memory_stats(dev)["used"]
+    srv = tc.Server(hbm_budget_bytes=budget, workers=2, max_batch=1 if room > 1 else 2, max_tick_pairs=1 << 30)
+    tickets = srv.submit_many(specs)
+    srv.drain(timeout_ms=300000)
+    res = {r["ticket"]: r for r in srv.poll()}
+    st = srv.stats()
+    srv.free()
+    real = tc.memory_stats(dev)["used_high"] - base
+    assert st["failed"] == 0
+    assert real <= st["peak_bytes_in_flight"] <= budget, (real, st["peak_bytes_in_flight"], budget)
+    for (seed, scale, _, _), t in zip(specs, tickets):
+        assert res[t]["triangles"] == standalone(tc, inputs.GraphSpec("rmat", seed, n, num_pairs=pairs, scale=scale))
+    with pytest.raises(tc.TCError) as ei:
+        srv = tc.Server(hbm_budget_bytes=footprint(specs[:1]) - 1, workers=1)
+        srv.submit_rmat(*specs[0])
+    srv.free()
+    assert ei.value.status == tc.TC_EBUSY
