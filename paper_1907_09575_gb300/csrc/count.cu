@@ -1259,11 +1259,19 @@ __global__ void __launch_bounds__(kMidThreads, kLightMinBlocks)
     GraphAcc acc;
     uint64_t probes = 0, staged = 0;
     unsigned long long nu = 0, nt = 0;
-    while (true) {
+    // The first of a list's units are dealt to the warps, the rest popped: a
+    // queue head serves its atomics one after the other, about 3 ns each, and a
+    // pop of each list and one more to find it empty were most of a count of some
+    // thousand units of 16 tasks (RMAT of 65,536 pairs and vertices: 30 us, 18
+    // dealt).  Warp units are dealt only where no warp has wide ones before them.
+    const long long all = (long long)gridDim.x * (kMidThreads / 32), me = (long long)w * gridDim.x + blockIdx.x;
+    auto pop = [&](int head, long long n, long long dealt, int step) {
+        if (dealt >= n) return n;
         long long u = 0;
-        if (lane == 0) u = (long long)atomicAdd(&ctr[CTR_MID_HEAD], 1ull);
-        u = __shfl_sync(0xffffffffu, u, 0);
-        if (u >= nunits) break;
+        if (lane == 0) u = (long long)atomicAdd(&ctr[head], (unsigned long long)step);
+        return dealt + __shfl_sync(0xffffffffu, u, 0);
+    };
+    for (long long u = me; u < nunits; u = pop(CTR_MID_HEAD, nunits, all, 1)) {
         const Unit U = units[u];
         const GraphView G = views[U.g];
         const int64_t rb = off_at(G, U.j);
@@ -1336,13 +1344,10 @@ __global__ void __launch_bounds__(kMidThreads, kLightMinBlocks)
     }
     // the warp units
     FlatWarp& S = *reinterpret_cast<FlatWarp*>(mine);
-    while (true) {
-        long long u0 = 0;
-        if (lane == 0) u0 = (long long)atomicAdd(&ctr[CTR_SMALL_HEAD], (unsigned long long)grab);
-        u0 = __shfl_sync(0xffffffffu, u0, 0);
-        if (u0 >= nsmall) break;
+    const long long dealt = nunits == 0 ? all * grab : 0;
+    for (long long u0 = dealt ? me * grab : pop(CTR_SMALL_HEAD, nsmall, 0, grab); u0 < nsmall;
+         u0 = pop(CTR_SMALL_HEAD, nsmall, dealt, grab))
         flat_units<PV>(views, small, u0, (int)min64(grab, nsmall - u0), S, cnt, tlow, acc, s_work[w]);
-    }
     acc.flush();
     __syncwarp();
     if (lane < 4 && s_work[w][0]) {
@@ -1607,9 +1612,11 @@ void launch_count_raw(const CountLaunch& c, const GraphView* views_dev, const Un
         TC_LAUNCH_CHECK();
     }
     if (c.light && L.nzone + L.nsmall > 0) {
-        // as many warp units at a time as leave every warp a turn
+        // as many warp units at a time as leave every warp a turn; up to
+        // kFlatUnits a warp, where they are dealt, so that nothing is popped
         const int64_t warps = (int64_t)num_sms() * kLightMinBlocks * (kMidThreads / 32);
-        const int grab = (int)std::max<int64_t>(1, std::min<int64_t>(kFlatUnits, L.nsmall / warps));
+        const int grab = (int)std::max<int64_t>(
+            1, std::min<int64_t>(kFlatUnits, (L.nsmall + (L.nzone == 0 ? warps - 1 : 0)) / warps));
         const int64_t items = L.nzone + (L.nsmall + grab - 1) / grab;
         const unsigned blocks = (unsigned)std::min<int64_t>((items + kMidThreads / 32 - 1) / (kMidThreads / 32),
                                                             (int64_t)num_sms() * kLightMinBlocks);

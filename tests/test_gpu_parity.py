@@ -398,3 +398,17 @@ def test_short_rows_searched(tc, pairs, merge):
     assert b.count().tolist() == [want, want]
     b.free()
     g.free()
+
+
+@pytest.mark.parametrize("k", [1, 31, 33, 4863, 4864, 4865, 9729, 14593, 19455, 19456, 19457, 40001])
+def test_units_dealt_and_popped(tc, k):
+    """k disjoint triangles are k warp units: fewer than the device's warps,
+    as many as they are dealt, and more."""
+    ids = np.random.default_rng(k).permutation(3 * k).astype(np.int32).reshape(k, 3)
+    s, d = ids[:, [0, 1, 2]].ravel(), ids[:, [1, 2, 0]].ravel()
+    g = tc.preprocess(torch.from_numpy(s.copy()).cuda(), torch.from_numpy(d.copy()).cuda(), 3 * k)
+    assert g.count() == k
+    total, t = g.count(per_vertex=True)
+    assert total == k and bool((t == 1).all())
+    assert g.count_stats()["units"] == [k, 0] and g.count_stats()["tasks"] == [k, 0]
+    g.free()
