@@ -135,3 +135,31 @@ def test_hashed_pivots_use_no_zones(tc, small_max):
     assert sum(g.count_stats()["probes"]) == hashed
     assert g.count(tuning=t) == want and sum(g.count_stats()["probes"]) == hashed
     g.free()
+
+
+@pytest.mark.parametrize("hubs,density", [(200, 0.9), (2047, 0.1), (2048, 0.1), (2049, 0.1), (2080, 0.1)])
+def test_zone_edges_with_zones(tc, hubs, density):
+    """The hubs' number around a zone's labels, in graphs of enough pairs to
+    have zones and with pivots that use them."""
+    want, names = launched(tc, lambda: check(tc, *hub_graph(hubs, 8000, 80, density, hubs)))
+    assert want > 0 and "k_zone" in names
+
+
+@pytest.mark.parametrize("tuning", [{"small_max_outdeg": 1}, {"slice_max": 64}, {"warp_unit_tasks": 1, "cta_unit_tasks": 1},
+                                    {"cta_threads": 64, "slice_max": 100, "merge_max_outdeg": 64},
+                                    {"cta_unit_tasks": 100000, "merge_max_outdeg": 8, "small_max_outdeg": 16}])
+def test_tunings_with_zones(tc, tuning):
+    hs, hd, n = hub_graph(2500, 8000, 80, 0.3, 4)
+    want, want_t = oracle.count(hs, hd, n, per_vertex=True)
+    t = tc.tuning_default()
+    for k, v in tuning.items():
+        setattr(t, k, v)
+    g = tc.preprocess(torch.from_numpy(hs).cuda(), torch.from_numpy(hd).cuda(), n)
+    (total, pv), names = launched(tc, lambda: g.count(per_vertex=True, tuning=t))
+    assert "k_zone" in names
+    assert total == want and np.array_equal(pv.cpu().numpy().astype(np.uint64), want_t)
+    assert g.count(tuning=t) == want
+    b = tc.Batch([g, g], tuning=t)
+    assert b.count().tolist() == [want, want]
+    b.free()
+    g.free()
