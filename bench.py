@@ -274,14 +274,14 @@ def traffic_for(kernel: str, workload: str, units: float, per_vertex: bool = Tru
     return per_unit * units, f"ncu capture of {c['case']} scaled by units ({c['unit_name']})"
 
 
-def alg_bytes_count(kstats: dict, off_bytes: int) -> float:
+def alg_bytes_count(kstats: dict, off_bytes: int, zone_probes: int = 0) -> float:
     """Algorithmic bytes of one count (all its kernels): per unit its record
     (32 B) and the pivot row bounds (2 offsets); per staged pivot entry 4 B;
-    per task its record (16 B); per probe the 4-B entry of U_i, also where the
-    entry is tested as one bit of a dense zone's block (fewer bytes are read
-    there).  Per-vertex flushes are not counted (atomics)."""
+    per task its record (16 B); per probe the 4-B entry of U_i, or a bit where
+    the entry is tested in a dense zone's block (whose other bits are read with
+    it and not counted).  Per-vertex flushes are not counted (atomics)."""
     return (sum(kstats["units"]) * (32 + 2 * off_bytes) + 4 * sum(kstats["staged"])
-            + 16 * sum(kstats["tasks"]) + 4 * sum(kstats["probes"]))
+            + 16 * sum(kstats["tasks"]) + 4 * (sum(kstats["probes"]) - zone_probes) + zone_probes / 8)
 
 
 # ----------------------------------------------------------------------------
@@ -500,6 +500,7 @@ def run_ours(args, wl):
     tc.profile_enable(False)
     count_ms = ev0.elapsed_time(ev1) / args.steps
     kst = g.count_stats()
+    zone_probes = g.zone_probes()
     g.free()
 
     # --- roofline of the dominant kernel of the step ---------------------
@@ -514,17 +515,19 @@ def run_ours(args, wl):
     kname, (klaunch, kms) = top
     roof = None
     if kname == "k_count":
-        b_launch = alg_bytes_count(kst, facts["offset_bytes"])
+        b_launch = alg_bytes_count(kst, facts["offset_bytes"], zone_probes)
         avg_ms = kms / klaunch
         achieved = b_launch / (avg_ms / 1e3) / 1e9
         traffic, tnote = traffic_for(kname, args.workload, sum(kst["probes"]), wl["per_vertex"])
-        roof = {"kernel": "+".join(parts), "bound": "hbm", "achieved": achieved, "peak": hbm,
+        # none of them is near a memory limit (profiles/): instructions bound them
+        roof = {"kernel": "+".join(parts), "bound": "issue", "achieved": achieved, "peak": hbm,
                 "unit": "GB/s", "frac": achieved / hbm, "traffic": traffic,
                 "traffic_note": tnote, "peak_source": peak_src,
                 "alg_bytes_per_launch": b_launch, "avg_launch_ms": avg_ms,
                 "share_of_step_kernel_time": kms / step_kernel_ms,
                 "kernels_ms": {k: v[1] / klaunch for k, v in parts.items()},
-                "probes_per_launch": sum(kst["probes"])}
+                "probes_per_launch": sum(kst["probes"]), "zone_probes_per_launch": zone_probes,
+                "gprobes_per_s": sum(kst["probes"]) / avg_ms / 1e6}
     else:
         roof = {"kernel": kname, "bound": "hbm", "achieved": None, "peak": hbm, "unit": "GB/s",
                 "frac": None, "traffic": None, "peak_source": peak_src,
@@ -725,13 +728,15 @@ def run_batch(args, wl):
 
     hbm, peak_src = peaks()
     kb = prof.get("k_count_batch", (args.steps, ms * args.steps))
-    b_launch = alg_bytes_count(kst, wl["offsets"] // 8)
+    zone_probes = sum(g.zone_probes() for g in graphs)
+    b_launch = alg_bytes_count(kst, wl["offsets"] // 8, zone_probes)
     achieved = b_launch / (kb[1] / kb[0] / 1e3) / 1e9
-    roof = {"kernel": "k_count (batched, one captured launch)", "bound": "hbm",
+    roof = {"kernel": "k_count+k_light+k_zone (batched, one captured launch)", "bound": "issue",
             "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
             "traffic": None, "traffic_note": "no ncu capture of the batched launch committed",
             "peak_source": peak_src, "alg_bytes_per_launch": b_launch,
-            "avg_launch_ms": kb[1] / kb[0]}
+            "avg_launch_ms": kb[1] / kb[0], "probes_per_launch": sum(kst["probes"]),
+            "zone_probes_per_launch": zone_probes, "gprobes_per_s": sum(kst["probes"]) / (kb[1] / kb[0]) / 1e6}
 
     e2e = None
     if not args.no_e2e:

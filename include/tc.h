@@ -299,6 +299,11 @@ typedef struct {
  * stream).  TC_EINVAL on NULL arguments; TC_ECUDA. */
 TC_API tc_status tc_count_get_stats(const tc_graph* g, tc_count_stats* out, void* stream);
 
+/* Of probes[1] of the graph's last tc_count, the entries that were bits of
+ * dense zones' blocks: read as such, not as 4-byte labels (0 for graphs without
+ * zones and with table_mode 1).  No device work.  TC_EINVAL on NULL arguments. */
+TC_API tc_status tc_count_get_zone_probes(const tc_graph* g, uint64_t* out);
+
 /* Fills *out with the graph's facts.  TC_EINVAL on NULL arguments. */
 TC_API tc_status tc_graph_get_stats(const tc_graph* g, tc_graph_stats* out);
 

@@ -113,9 +113,10 @@ void tuning_resolve(const tc_tuning* in, tc_tuning* out) {
     out->merge_max_outdeg = std::max(0, std::min(in->merge_max_outdeg, out->small_max_outdeg));
 }
 
-// Warp units of 16 tasks spread a small graph's few units over the SMs
-// (RMAT scale 14: 87 -> 48 us per count); from 2^21 edges up 64 are as fast
-// or faster (scale 20: 1.87 ms either way; scale 26: 426 against 429 ms).
+// Warp units of 16 tasks spread a small graph's few units over the SMs; searched
+// four at a time they differ little from 64 (RMAT of 2^18 pairs, 4 a vertex: 56
+// and 59 us; mostly equal below), and from 2^21 edges up 64 are as fast or
+// faster (G(n,p) of 2^22 pairs, 16 a vertex: 165 and 148 us; RMAT alike).
 tc_tuning size_tuning(const tc_tuning& t, int64_t m) {
     tc_tuning out = t;
     if (out.warp_unit_tasks <= 0) out.warp_unit_tasks = m < (1ll << 21) ? 16 : 64;
@@ -456,6 +457,13 @@ tc_status tc_count_get_stats(const tc_graph* g, tc_count_stats* out, void* strea
         out->staged[k] = c[CTR_STAGED + k];
     }
     out->probes[1] += g->zone_probes;
+    TC_API_END
+}
+
+tc_status tc_count_get_zone_probes(const tc_graph* g, uint64_t* out) {
+    TC_API_BEGIN
+    if (!g || !out) TC_FAIL(TC_EINVAL, "tc_count_get_zone_probes: NULL argument");
+    *out = g->zone_probes;
     TC_API_END
 }
 

@@ -1397,7 +1397,8 @@ __global__ void k_unit_counts(const GraphView* __restrict__ views, const int64_t
         const GraphView& G = views[g];
         const int64_t j = v - vpre[g];
         int64_t a, b, c;
-        unit_split<true>(rule, rule.zones && G.zrow != nullptr, off_at(G, j + 1) - off_at(G, j), G.loff[j + 1] - G.loff[j], a, b, c);
+        unit_split<true>(rule, rule.zones && G.zrow != nullptr, off_at(G, j + 1) - off_at(G, j),
+                         G.loff[j + 1] - G.loff[j], a, b, c);
         cs[x] = (int32_t)a;
         cl[x] = (int32_t)b;
         if (cz) cz[x] = (int32_t)c;

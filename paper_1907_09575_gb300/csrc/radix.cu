@@ -151,8 +151,8 @@ __global__ void __launch_bounds__(kRadix) k_digit_offsets(unsigned long long* __
 // What bounds it is instructions and the look-back: 16 B of traffic a key is
 // 2.5 ms of a 2^30-key pass; staged in shared memory, ranked there and looked
 // back one tile at a time the pass took 7.2 ms, 170 instructions for every 32
-// keys.  So a key stays in its thread's registers from the load to its place
-// in the tile (warp w holds a contiguous segment, a row of 32 keys a
+// keys.  So a key stays with its thread from the load to its place in the tile,
+// in registers but for 116 bytes (three blocks an SM leave 80 registers a thread) (warp w holds a contiguous segment, a row of 32 keys a
 // register), its rank beside it, two to a register; a digit's place in the
 // output is one 64-bit word, to which the key's place in the tile is added;
 // the look-back reads kLook tiles' words at a time, and the keys move to their

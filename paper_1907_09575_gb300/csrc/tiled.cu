@@ -152,7 +152,7 @@ void graph_offload(tc_graph* g, cudaStream_t st) {
     g->zbits = g->zowner = nullptr;
     g->zrow = nullptr;
     g->zcap = 0;
-    g->covered = 0;
+    g->covered = g->zone_probes = 0;
     g->units_bytes = g->arena_bytes = g->tlow_bytes = 0;
     g->units_tuning = tc_tuning{};
     g->host = h;

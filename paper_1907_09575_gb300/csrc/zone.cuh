@@ -42,8 +42,8 @@ constexpr int kZoneTasks = 248;       // tasks of one unit of the zone kernel: a
 // for none.  No zones, and no pivots of more than 64 entries for single warps,
 // up to 2^19 edges: there a count is as long as its longest unit, which eight
 // warps share, and the further launches cost what they save (kept RMAT graphs,
-// totals: 2^17 pairs 45 us as CTA units, 60 by warps; 2^18 65 and 75; 2^19 81
-// and 96 with zones; 2^20 132 and 110).
+// totals: 2^17 pairs 30 us as CTA units, 52 by warps with zones; 2^18 47 and
+// 69; 2^19 63 and 76; 2^20 106 and 92; 2^21 196 and 121).
 // A graph preprocessed in one launch has them by its pairs, which the host
 // knows before its edges: zcap, not m, says whether a graph has zones.
 inline bool zones_at(int64_t m) { return m > (1ll << 19); }

@@ -70,7 +70,7 @@ EXPORTS = ("tc_preprocess", "tc_count", "tc_triangles", "tc_graph_get_stats", "t
            "tc_server_create", "tc_server_now", "tc_server_submit_rmat", "tc_server_poll",
            "tc_server_drain", "tc_server_get_stats", "tc_server_free", "tc_release_memory",
            "tc_selftest_wait_timeout", "tc_server_submit_rmat_many", "tc_memory_get_stats",
-           "tc_triangles_get_timing", "tc_graph_offload", "tc_count_tiled")
+           "tc_triangles_get_timing", "tc_graph_offload", "tc_count_tiled", "tc_count_get_zone_probes")
 
 TC_STATIC_MAX_PAIRS = 262144
 TC_STATIC_MAX_VERTICES = 65536
@@ -164,6 +164,8 @@ def load(path: str = LIB_PATH) -> ctypes.CDLL:
     lib.tc_generate_rmat.restype = st
     lib.tc_count_get_stats.argtypes = [vp, ctypes.POINTER(CountStats), vp]
     lib.tc_count_get_stats.restype = st
+    lib.tc_count_get_zone_probes.argtypes = [vp, ctypes.POINTER(ctypes.c_uint64)]
+    lib.tc_count_get_zone_probes.restype = st
     lib.tc_server_create.argtypes = [ctypes.POINTER(ServerConfig), ctypes.POINTER(vp)]
     lib.tc_server_create.restype = st
     lib.tc_server_now.argtypes = [vp]
@@ -324,6 +326,13 @@ class Graph:
         _check(load().tc_count_get_stats(self._h, ctypes.byref(c), _stream_ptr(stream)))
         return {"triangles": int(c.triangles), "units": list(c.units), "tasks": list(c.tasks),
                 "probes": list(c.probes), "staged": list(c.staged)}
+
+    def zone_probes(self) -> int:
+        """Of the last count's probes, those tested as bits of dense zones
+        (tc_count_get_zone_probes)."""
+        z = ctypes.c_uint64(0)
+        _check(load().tc_count_get_zone_probes(self._h, ctypes.byref(z)))
+        return int(z.value)
 
     def count(self, per_vertex=None, total_dev=None, tuning: Optional[Tuning] = None,
               stream=None, sync: bool = True):

@@ -126,13 +126,14 @@ def test_hashed_pivots_use_no_zones(tc, small_max):
     assert total == want and np.array_equal(pv.cpu().numpy().astype(np.uint64), want_t)
     assert not names & {"k_zone", "k_light"}, names
     hashed = sum(g.count_stats()["probes"])
+    assert g.zone_probes() == 0
     b = tc.Batch([g, g], tuning=t)
     assert b.count().tolist() == [want, want]
     assert sum(b.count_stats()["probes"]) == 2 * hashed
     b.free()
     total, names = launched(tc, g.count)
     assert total == want and {"k_zone", "k_light"} <= names
-    assert sum(g.count_stats()["probes"]) == hashed
+    assert sum(g.count_stats()["probes"]) == hashed and 0 < g.zone_probes() < hashed
     assert g.count(tuning=t) == want and sum(g.count_stats()["probes"]) == hashed
     g.free()
 
