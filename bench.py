@@ -527,7 +527,9 @@ def run_ours(args, wl):
                 "share_of_step_kernel_time": kms / step_kernel_ms,
                 "kernels_ms": {k: v[1] / klaunch for k, v in parts.items()},
                 "probes_per_launch": sum(kst["probes"]), "zone_probes_per_launch": zone_probes,
-                "gprobes_per_s": sum(kst["probes"]) / avg_ms / 1e6}
+                "gprobes_per_s": sum(kst["probes"]) / avg_ms / 1e6,
+                # adjacency entries at 4 B each whatever the form they are tested in
+                "adjacency_frac": 4 * sum(kst["probes"]) / (avg_ms / 1e3) / 1e9 / hbm}
     else:
         roof = {"kernel": kname, "bound": "hbm", "achieved": None, "peak": hbm, "unit": "GB/s",
                 "frac": None, "traffic": None, "peak_source": peak_src,

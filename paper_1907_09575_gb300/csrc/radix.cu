@@ -151,16 +151,17 @@ __global__ void __launch_bounds__(kRadix) k_digit_offsets(unsigned long long* __
 // What bounds it is instructions and the look-back: 16 B of traffic a key is
 // 2.5 ms of a 2^30-key pass; staged in shared memory, ranked there and looked
 // back one tile at a time the pass took 7.2 ms, 170 instructions for every 32
-// keys.  So a key stays with its thread from the load to its place in the tile,
-// in registers but for 116 bytes (three blocks an SM leave 80 registers a thread) (warp w holds a contiguous segment, a row of 32 keys a
-// register), its rank beside it, two to a register; a digit's place in the
-// output is one 64-bit word, to which the key's place in the tile is added;
-// the look-back reads kLook tiles' words at a time, and the keys move to their
-// places before it starts (2^30 keys: 7.2 -> 5.7 ms; 1, 2, 4, 8 words: 6.0,
-// 5.9, 5.7, 5.8).  Larger tiles share out a tile's fixed work -- counters, scan,
-// look-back -- further: 16, 24, 26, 28 keys a thread 4.9, 4.6, 4.5, 4.5 ms
-// (the first at four blocks an SM, the others at three).  The last tile is filled up with keys of the highest digit,
-// which end up behind its own and are not written.
+// keys.  So a key stays with its thread from the load to its place in the tile
+// (in registers but for 116 bytes: three blocks an SM leave 80 a thread; warp w
+// holds a contiguous segment, a row of 32 keys a register), its rank beside it,
+// two to a register; a digit's place in the output is one 64-bit word, to which
+// the key's place in the tile is added; the look-back reads kLook tiles' words
+// at a time, and the keys move to their places before it starts (2^30 keys: 7.2
+// -> 5.7 ms; 1, 2, 4, 8 words: 6.0, 5.9, 5.7, 5.8).  Larger tiles share out a
+// tile's fixed work -- counters, scan, look-back -- further: 16, 24, 26, 28 keys
+// a thread 4.9, 4.6, 4.5, 4.5 ms (the first at four blocks an SM, the others at
+// three).  The last tile is filled up with keys of the highest digit, which end
+// up behind its own and are not written.
 #ifndef TC_SWEEP_MINB
 #define TC_SWEEP_MINB 3
 #endif
