@@ -869,16 +869,16 @@ void graph_views(const tc_graph* g, GraphView* v, GraphView* vc) {
 
 // Preprocessing in one launch sizes the arena by the pairs and the units by
 // their bound.  A graph that is kept moves to what its edges need when it holds
-// over half as much again, and 8 MiB: pairs given many times, or few pairs a
-// vertex (RMAT scale 14, 65,536 pairs 64 times: 93.1 MB -> 2.0; scale 20 of
-// 2^20 pairs: 97.4 -> 61.2).
+// over twice that, and 8 MiB more: pairs given many times (RMAT scale 14, 65,536
+// pairs 64 times: 93.1 MB -> 2.0).  Graphs whose pairs are mostly edges hold up
+// to 1.6 times their need and stay.
 void graph_trim(tc_graph* g, cudaStream_t st) {
     if (!g->arena || !g->units_mem) return;
     const int64_t units = std::max<int64_t>(g->n_large + g->n_zone + g->n_small, 1);
     const int64_t zcap = g->zcap > 0 ? std::min(g->zcap, g->zone_blocks + 1) : 0;
     const size_t held = g->arena_bytes + g->units_bytes;
     const size_t need = ArenaPlan(g->n, g->m, zcap, g->off64, g->num_comps).bytes + sizeof(Unit) * (size_t)units;
-    if (held < need + std::max<size_t>(need / 2, 8 << 20)) return;
+    if (held < need + std::max<size_t>(need, 8 << 20)) return;
     const tc_graph old = *g;
     UnitLists L = units_of(g);
     L.mem = nullptr;

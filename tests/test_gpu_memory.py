@@ -120,8 +120,8 @@ def repeated_pairs(tc, kind):
 @pytest.mark.parametrize("kind", ["one", "small", "zones"])
 @pytest.mark.parametrize("offsets", [None, 64])
 def test_kept_graph_holds_what_its_edges_need(tc, kind, offsets):
-    """A graph that stays holds at most half as much again as its edges need
-    (and 8 MiB), however often its pairs were given, and counts the same."""
+    """A graph that stays holds at most twice what its edges need (and 8 MiB),
+    however often its pairs were given, and counts the same."""
     (s, d, n), (s1, d1, _) = repeated_pairs(tc, kind)
     once = tc.preprocess(s1, d1, n, offsets=offsets)
     want, want_t = once.count(per_vertex=True)
@@ -129,7 +129,7 @@ def test_kept_graph_holds_what_its_edges_need(tc, kind, offsets):
     g = tc.preprocess(s, d, n, offsets=offsets)
     torch.cuda.synchronize()
     held = tc.memory_stats(torch.cuda.current_device())["used"] - used
-    assert held <= 1.5 * once.stats()["device_bytes"] + (9 << 20), (held, once.stats())
+    assert held <= 2 * once.stats()["device_bytes"] + (9 << 20), (held, once.stats())
     assert g.stats()["device_bytes"] <= held
     assert g.stats()["m"] == once.stats()["m"]
     total, t = g.count(per_vertex=True)
