@@ -83,7 +83,8 @@ typedef struct {
                                   traversal of Section 3.1), or, with many tasks, the
                                   pivot gets a table per warp */
     int32_t warp_unit_tasks;   /* tasks per warp unit (<= 8192); 0: 16 for graphs of
-                                  fewer than 2^21 edges, else 64 */
+                                  fewer than 2^21 edges (pairs, up to 2^22 of them),
+                                  else 64 */
     int32_t cta_unit_tasks;    /* tasks per CTA unit (<= 8192) */
     int32_t cta_threads;       /* threads per CTA of the large-pivot kernel (64..256);
                                   pivots of 65 to 256 entries are counted by single
